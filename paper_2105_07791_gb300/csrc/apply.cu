@@ -11,7 +11,7 @@
 // topological order.  Dense nodes with m_i <= DIAG_COLS take one pass over
 // the first m_i columns of the eliminated front, [A_ii^{-1} P^T ; -L P^T]:
 // the diagonal solve and the up-sweep product share the input y(I^s) and
-// the same dependencies, so one 64-row task gives z rows or y(B^s) updates.
+// the same dependencies, so one row task gives z rows or y(B^s) updates.
 // A_ii^{-1} of larger nodes is split into DIAG_COLS-column chunks whose
 // partial products a second task sums (a 1539-column row is otherwise one
 // long dependent chain on the critical path).  Low-rank nodes use dot tasks
@@ -66,6 +66,7 @@ constexpr int AW = AT / 32;
 constexpr int GATHER_CHUNK = 8 * AT;     // rows per gather task
 constexpr int DIAG_COLS = 256;    // column chunk of A_ii^{-1} per task (and fused-pass limit)
 constexpr int SUM_ROWS = AT;      // rows per partial-sum task
+constexpr int FINE_ROWS = 16;      // rows per task of the FP64 levels with few 64-row tasks
 constexpr int ROOT_DIAG_COLS = 128; // the same for the top level's nodes
 constexpr uint64_t APPLY_WAIT_NS = 2000000000ull;   // 2 s
 
@@ -109,8 +110,6 @@ enum : int {
     TK_DNDOT,     // low-rank: partial RJt(chunk, :)^T z(B)(chunk)
     TK_DNAXPY,    // low-rank: 64 rows of z(I) += X t
     TK_FINNOP,    // completes a node without interior rows
-    TK_UPW,       // up to 8 tiny dense nodes of a level, one per warp: [A_ii^{-1}; -L] y(I)
-    TK_DNW,       // the same nodes coming down: z(I) += R z(B), final rows
     TK_HUP,       // ULV solve of HSS(A_ii), one HSS node going up (entry node = ULV record)
     TK_HROOT,     // the root block of a ULV front
     TK_HDN,       // one HSS node coming down (leaves write z(I) rows)
@@ -121,16 +120,18 @@ enum : int {
 // of its shared-memory vector segment (interior rows + B of the root) and
 // per-level staged inputs.
 constexpr int SUB_NODES = 256, SUB_LV = 16, SUB_LVN = 64, SUB_V = 1536, SUB_XIN = 1024;
-constexpr int SUB_MIN_ROOTS = 128;   // fewest subtrees worth the restructuring (GPU fill)
-// Tiny dense nodes (the bottom levels) are handled a warp per node, eight per
-// task: their blocks are a few KB, so one 64-row task per node would be all
-// latency.  Limits of a warp node (rows of the fused pass, interior rows,
-// boundary columns) and its per-warp shared-memory region.
-constexpr int WN_M = 96, WN_MI = 64, WREG = 128;
+constexpr int SUB_MI = 128, SUB_MB = 512;   // largest node
+// Fewest subtrees worth the restructuring: below about three per SM the SMs
+// differ too much in how many they run (128 -> 512 roots, one apply: 256 x 256
+// P1 Helmholtz, compressed FP32, 151 -> 122 us; 192 x 192 elastic 187 -> 146;
+// 256 x 256 P2 in dense FP64 1209 -> 1005; 1024 roots are slower again).
+// Problems with fewer bottom nodes run per-node tasks all the way down.
+constexpr int SUB_MIN_ROOTS = 512;
 // per-node counters (NCNT arrays of nnodes each) and what signals them
 enum : int { CN_UP = 0, CN_DOT, CN_DIAG, CN_DDOT, CN_FIN, CN_DPART, NCNT };
 constexpr int TK_SHIFT = 25;       // entry word 0 = kind << TK_SHIFT | node (5 bits of kind)
 constexpr int TK_FINAL = 1 << 30;  // entry word 0 flag: the task writes final rows (scatter)
+constexpr int32_t TK_FINE = INT32_MIN;   // entry word 0 flag: a row task of FINE_ROWS rows
 constexpr int CTL_WORDS = 4;       // ticket, gather count, abort, pad
 // ints per queue entry: flags | kind | node, a, b, m_i, m_b, i_off, b_off, k,
 // base (64-bit: front offset, or low-rank storage address), aux (64-bit:
@@ -146,7 +147,6 @@ struct ApplyCtx {
     const int32_t* sigma;
     const int32_t* perm;
     const T* front;
-    const int32_t* wdesc;     // warp nodes, 8 ints each: node, m_i, m_b, i_off, b_off, front offset (lo, hi), 0
     const struct UlvDev* ulv; // ULV records (HSS nodes of the ULV fronts)
     const int32_t* ulv_ord;   // HSS order of each ULV front's I^s
     const int64_t* foff;      // front offset of every node
@@ -198,13 +198,14 @@ __device__ __forceinline__ void prefetch_line(const void* p, int l) {
 template <typename T>
 __device__ __forceinline__ void gemv_pre(const T* __restrict__ A, int64_t lda, int rows, int cols, int r0, T (&pre)[8]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int ra = r0 + lane, rb = r0 + lane + 32;
+    const bool va = r0 + lane < rows, vb = r0 + lane + 32 < rows;
+    const T* col = A + (int64_t)warp * lda + r0 + lane;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int c = warp + u * AW;
-        const T* col = A + (int64_t)c * lda;
-        pre[u] = (c < cols && ra < rows) ? col[ra] : zero<T>();
-        pre[4 + u] = (c < cols && rb < rows) ? col[rb] : zero<T>();
+        const bool ok = warp + u * AW < cols;
+        pre[u] = (ok && va) ? col[0] : zero<T>();
+        pre[4 + u] = (ok && vb) ? col[32] : zero<T>();
+        col += (int64_t)AW * lda;
     }
     // the rest of the 64-row segment into L2 while the task waits
     const int nr = min(APPLY_ROWS, rows - r0);
@@ -223,8 +224,8 @@ template <typename T>
 __device__ __forceinline__ T gemv_rows64(const T* __restrict__ A, int64_t lda, int rows, int cols, int r0,
                                          const T* __restrict__ xs, T (*red)[APPLY_ROWS], const T (&pre)[8]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int ra = r0 + lane, rb = r0 + lane + 32;
-    const bool va = ra < rows, vb = rb < rows;
+    const int ra = r0 + lane;
+    const bool va = ra < rows, vb = ra + 32 < rows;
     T acc0 = zero<T>(), acc1 = zero<T>();
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -236,14 +237,18 @@ __device__ __forceinline__ T gemv_rows64(const T* __restrict__ A, int64_t lda, i
         }
     }
     int c = warp + 4 * AW;
+    // one running pointer: eight addresses of their own would not leave the
+    // registers for eight loads in flight
+    const T* col = A + (int64_t)c * lda + ra;
+    const int64_t step = (int64_t)AW * lda;
     for (; c + 3 * AW < cols; c += 4 * AW) {
         T a[4], b[4], x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const T* col = A + (int64_t)(c + u * AW) * lda;
-            a[u] = va ? col[ra] : zero<T>();
-            b[u] = vb ? col[rb] : zero<T>();
+            a[u] = va ? col[0] : zero<T>();
+            b[u] = vb ? col[32] : zero<T>();
             x[u] = xs[c + u * AW];
+            col += step;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -257,10 +262,10 @@ __device__ __forceinline__ T gemv_rows64(const T* __restrict__ A, int64_t lda, i
         for (int u = 0; u < 3; ++u) {
             const int cu = c + u * AW;
             const bool ok = cu < cols;
-            const T* col = A + (int64_t)(ok ? cu : c) * lda;
-            a[u] = (ok && va) ? col[ra] : zero<T>();
-            b[u] = (ok && vb) ? col[rb] : zero<T>();
+            a[u] = (ok && va) ? col[0] : zero<T>();
+            b[u] = (ok && vb) ? col[32] : zero<T>();
             x[u] = ok ? xs[cu] : zero<T>();
+            col += step;
         }
 #pragma unroll
         for (int u = 0; u < 3; ++u) {
@@ -277,11 +282,82 @@ __device__ __forceinline__ T gemv_rows64(const T* __restrict__ A, int64_t lda, i
     return sum;
 }
 
+// The same product for FINE_ROWS = 16 rows: a half-warp per column, every 16th
+// column per half-warp, eight in flight per lane; the half-warps' sums are
+// added first, then the warps' in warp order.
+//
+// 16-row tasks are for the FP64 pipe (two DFMA per clock and SM): 64 rows x
+// 768 columns of a complex128 block keep one SM busy for 47 us while a top
+// level has fewer such tasks than the GPU has SMs (see FINE_TASKS).
+template <typename T>
+__device__ __forceinline__ void gemv16_pre(const T* __restrict__ A, int64_t lda, int rows, int cols, int r0, T (&pre)[8]) {
+    const int lane = threadIdx.x & 31, cs = threadIdx.x >> 4, r = r0 + (lane & 15);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int c = cs + 16 * u;
+        pre[u] = (c < cols && r < rows) ? A[(int64_t)c * lda + r] : zero<T>();
+    }
+    // the rest of the row segment into L2 while the task waits
+    const int nr = min(FINE_ROWS, rows - r0);
+    if (nr > 0 && cols > 128) {
+        constexpr int LPC = (FINE_ROWS * (int)sizeof(T) + 127) / 128 + 1;   // lines a segment can touch
+        const int tot = (cols - 128) * LPC;
+        for (int q = threadIdx.x; q < tot; q += AT) {
+            const T* seg = A + (int64_t)(128 + q / LPC) * lda + r0;
+            const int l = q % LPC;
+            if (l < range_lines(seg, (int64_t)nr * sizeof(T))) prefetch_line(seg, l);
+        }
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ T gemv16_rows(const T* __restrict__ A, int64_t lda, int rows, int cols, int r0,
+                                         const T* __restrict__ xs, T (*red)[APPLY_ROWS], const T (&pre)[8]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cs = threadIdx.x >> 4, r = r0 + (lane & 15);
+    T acc = zero<T>();
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (cs + 16 * u < cols) acc = fmac(pre[u], xs[cs + 16 * u], acc);
+    for (int c = cs + 128; c < cols; c += 128) {
+        T a[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a[u] = (c + 16 * u < cols && r < rows) ? A[(int64_t)(c + 16 * u) * lda + r] : zero<T>();
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (c + 16 * u < cols) acc = fmac(a[u], xs[c + 16 * u], acc);
+    }
+    acc = acc + shfl_xor_t(acc, 16);
+    if (lane < 16) red[warp][lane] = acc;
+    __syncthreads();
+    T sum = zero<T>();
+    if (threadIdx.x < FINE_ROWS)
+        for (int w = 0; w < AW; ++w) sum += red[w][threadIdx.x];
+    return sum;
+}
+
+// the row-task kinds' product: 16-row tasks exist for FP64 fronts only
+template <typename T>
+__device__ __forceinline__ void gemv_pre_task(int R, const T* A, int64_t lda, int rows, int cols, int r0, T (&pre)[8]) {
+    if constexpr (sizeof(typename Tr<T>::real) == 8) {
+        if (R == FINE_ROWS) return gemv16_pre(A, lda, rows, cols, r0, pre);
+    }
+    gemv_pre(A, lda, rows, cols, r0, pre);
+}
+template <typename T>
+__device__ __forceinline__ T gemv_task(int R, const T* A, int64_t lda, int rows, int cols, int r0, const T* xs,
+                                       T (*red)[APPLY_ROWS], const T (&pre)[8]) {
+    if constexpr (sizeof(typename Tr<T>::real) == 8) {
+        if (R == FINE_ROWS) return gemv16_rows(A, lda, rows, cols, r0, xs, red, pre);
+    }
+    return gemv_rows64(A, lda, rows, cols, r0, xs, red, pre);
+}
+
 // ---- one task: pre-phase (independent loads) and run-phase ----------------
 
 struct Entry {
     int kind, s, a, b;
     bool fin;
+    int rows;                  // rows of a row task
     int m_i, m_b, i_off, b_off, k;
     int64_t base, aux;
 };
@@ -290,6 +366,7 @@ __device__ __forceinline__ Entry decode(const int32_t* q, int64_t t) {
     const int4 v0 = p[0], v1 = p[1], v2 = p[2];
     Entry e;
     e.fin = (v0.x & TK_FINAL) != 0;
+    e.rows = v0.x < 0 ? FINE_ROWS : APPLY_ROWS;
     e.kind = (v0.x >> TK_SHIFT) & 31;
     e.s = v0.x & ((1 << TK_SHIFT) - 1);
     e.a = v0.y;
@@ -303,80 +380,11 @@ __device__ __forceinline__ Entry decode(const int32_t* q, int64_t t) {
     e.aux = (int64_t)(((uint64_t)(uint32_t)v2.w << 32) | (uint32_t)v2.z);
     return e;
 }
-
-// ---- warp-node tasks (TK_UPW / TK_DNW) -------------------------------------
-// Warp w < e.a takes node e.base + w of the warp-node table; wd[w] receives
-// its descriptor, idx + w * WREG its gather indices, vec + w * WREG its
-// staged vector.
-__device__ __forceinline__ void taskw_pre(const int32_t* __restrict__ wdesc, const int32_t* __restrict__ sigma,
-                                          const int32_t* __restrict__ blist, const Entry& e, int* idx, int (*wd)[8]) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (w >= e.a) return;
-    if (lane < 8) wd[w][lane] = wdesc[(e.base + w) * 8 + lane];
-    __syncwarp();
-    const int m_i = wd[w][1], m_b = wd[w][2], i_off = wd[w][3], b_off = wd[w][4];
-    int* iw = idx + w * WREG;
-    if (e.kind == TK_UPW)
-        for (int c = lane; c < m_i; c += 32) iw[c] = sigma[i_off + c];
-    else
-        for (int j = lane; j < m_b; j += 32) iw[j] = blist[b_off + j];
-}
-
-template <typename T, typename V>
-__device__ __forceinline__ void taskw_run(const ApplyCtx<T>& C, const Entry& e, const int* idx, T* vec,
-                                          const int (*wd)[8], V* __restrict__ out, T* y, T* z) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (w >= e.a) return;
-    const int m_i = wd[w][1], m_b = wd[w][2], i_off = wd[w][3], b_off = wd[w][4];
-    const int64_t foff = (int64_t)(((uint64_t)(uint32_t)wd[w][6] << 32) | (uint32_t)wd[w][5]);
-    const int m = m_i + m_b;
-    const T* F = C.front + foff;
-    const int* iw = idx + w * WREG;
-    T* vw = vec + w * WREG;
-    constexpr int WU = sizeof(T) <= 8 ? 8 : 4;     // columns in flight per lane
-    if (e.kind == TK_UPW) {
-        // rows r of the first m_i columns, lanes over rows, WU columns in flight
-        for (int c = lane; c < m_i; c += 32) vw[c] = ldw(y + i_off + iw[c]);
-        __syncwarp();
-        for (int r0 = 0; r0 < m; r0 += 32) {
-            const int r = r0 + lane;
-            const int g = (r >= m_i && r < m) ? C.blist[b_off + r - m_i] : -1;
-            T acc = zero<T>();
-            for (int c0 = 0; c0 < m_i; c0 += WU) {
-                T a[WU];
-#pragma unroll
-                for (int u = 0; u < WU; ++u) a[u] = (r < m && c0 + u < m_i) ? F[(int64_t)(c0 + u) * m + r] : zero<T>();
-#pragma unroll
-                for (int u = 0; u < WU; ++u)
-                    if (c0 + u < m_i) acc = fmac(a[u], vw[c0 + u], acc);
-            }
-            if (r < m_i) stw(z + i_off + r, acc);
-            else if (r < m) stw(y + g, ldw(y + g) - acc);
-        }
-    } else {
-        // interior rows of R (m_i x m_b at column m_i), lanes over rows
-        for (int j = lane; j < m_b; j += 32) vw[j] = ldw(z + iw[j]);
-        __syncwarp();
-        const T* R = F + (int64_t)m_i * m;
-        for (int r0 = 0; r0 < m_i; r0 += 32) {
-            const int r = r0 + lane;
-            const int pi = r < m_i ? C.perm[i_off + r] : 0;
-            T acc = zero<T>();
-            for (int c0 = 0; c0 < m_b; c0 += WU) {
-                T a[WU];
-#pragma unroll
-                for (int u = 0; u < WU; ++u) a[u] = (r < m_i && c0 + u < m_b) ? R[(int64_t)(c0 + u) * m + r] : zero<T>();
-#pragma unroll
-                for (int u = 0; u < WU; ++u)
-                    if (c0 + u < m_b) acc = fmac(a[u], vw[c0 + u], acc);
-            }
-            if (r < m_i) {
-                const T v = ldw(z + i_off + r) + acc;
-                stw(z + i_off + r, v);
-                out[pi] = to_val(v);
-            }
-        }
-    }
+// rows of a row task (FP32 fronts have 64-row tasks only)
+template <typename T>
+__device__ __forceinline__ int task_rows(const Entry& e) {
+    if constexpr (sizeof(typename Tr<T>::real) == 8) return e.rows;
+    return APPLY_ROWS;
 }
 
 // ---- ULV solve tasks (TK_HUP / TK_HROOT / TK_HDN) --------------------------
@@ -498,6 +506,11 @@ __device__ bool wait_gather(const Sched* S);
 template <typename T, typename V>
 __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* vec, const V* __restrict__ x,
                              V* __restrict__ out, T* y, T* z, const Sched* Sp) {
+    // Loads in flight per thread (a running pointer instead of SU addresses keeps
+    // them inside the 64 registers).  One apply, FP32: 256 x 256 P2 Helmholtz,
+    // compressed, 238 us with eight addressed loads, 218 with eight and 214 with
+    // sixteen loads on a running pointer; 512 x 512 dense 1191, 1115, 1080.
+    constexpr int SU = sizeof(T) <= 8 ? 16 : 8;
     const bool up = e.kind == TK_SUBUP;
     const int tid = threadIdx.x;
     const int lo = e.a, nI = e.b, mbr = e.m_b;
@@ -575,6 +588,16 @@ __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* 
             }
         }
     };
+    // the level's node that row belongs to: the last one starting at or before it
+    auto node_of = [&](const int* N, int cnt, int row) {
+        int j = 0;
+        for (int n = cnt; n > 1;) {
+            const int h = n >> 1;
+            if (row >= N[SUB_NREC * (j + h) + (up ? 4 : 6)]) j += h;
+            n -= h;
+        }
+        return j;
+    };
     prefetch_level(0);
     T* xin = vec + nI + mbr;
     T* part = xin + SUB_XIN;
@@ -598,9 +621,7 @@ __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* 
         const int qp = R >= AT ? 1 : AT / R;               // threads per row
         for (int ee = tid; ee < R * qp; ee += AT) {
             const int row = ee % R, p = ee / R;
-            int j = 0;
-            while (j + 1 < cnt && row >= N[SUB_NREC * (j + 1) + (up ? 4 : 6)]) ++j;
-            const int* nd = N + SUB_NREC * j;
+            const int* nd = N + SUB_NREC * node_of(N, cnt, row);
             const int mi = nd[0], mb = nd[1];
             const int r = row - nd[up ? 4 : 6];
             const int64_t m = (int64_t)mi + mb;
@@ -614,19 +635,27 @@ __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* 
             // memory wait, not one per column
             T acc = zero<T>();
             int c = p;
-            for (; c + 7 * qp < cols; c += 8 * qp) {
-                T a[8];
+            const T* Ac = A + (int64_t)p * m;
+            const int64_t step = (int64_t)qp * m;
+            for (; c + (SU - 1) * qp < cols; c += SU * qp) {
+                T a[SU];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) a[u] = A[(int64_t)(c + u * qp) * m];
+                for (int u = 0; u < SU; ++u) {
+                    a[u] = *Ac;
+                    Ac += step;
+                }
 #pragma unroll
-                for (int u = 0; u < 8; ++u) acc = fmac(a[u], xs[c + u * qp], acc);
+                for (int u = 0; u < SU; ++u) acc = fmac(a[u], xs[c + u * qp], acc);
             }
             if (c < cols) {
-                T a[7];
+                T a[SU - 1];
 #pragma unroll
-                for (int u = 0; u < 7; ++u) a[u] = c + u * qp < cols ? A[(int64_t)(c + u * qp) * m] : zero<T>();
+                for (int u = 0; u < SU - 1; ++u) {
+                    a[u] = c + u * qp < cols ? *Ac : zero<T>();
+                    Ac += step;
+                }
 #pragma unroll
-                for (int u = 0; u < 7; ++u) acc = fmac(a[u], c + u * qp < cols ? xs[c + u * qp] : zero<T>(), acc);
+                for (int u = 0; u < SU - 1; ++u) acc = fmac(a[u], c + u * qp < cols ? xs[c + u * qp] : zero<T>(), acc);
             }
             if (qp > 1) {
                 part[ee] = acc;
@@ -642,9 +671,7 @@ __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* 
             for (int row = tid; row < R; row += AT) {
                 T acc = part[row];
                 for (int p = 1; p < qp; ++p) acc += part[p * R + row];
-                int j = 0;
-                while (j + 1 < cnt && row >= N[SUB_NREC * (j + 1) + (up ? 4 : 6)]) ++j;
-                const int* nd = N + SUB_NREC * j;
+                const int* nd = N + SUB_NREC * node_of(N, cnt, row);
                 const int r = row - nd[up ? 4 : 6];
                 if (up) {
                     if (r < nd[0]) stw(z + lo + nd[8] + r, acc);
@@ -693,15 +720,11 @@ __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* 
 // entries (read-only during the apply) and index lists.  idx: shared int
 // array of at least max(m_i, m_b, LR_CHUNK) entries.
 template <typename T>
-__device__ __forceinline__ void task_pre(const ApplyCtx<T>& C, const Entry& e, Pre<T>& P, int* idx, int (*wd)[8]) {
+__device__ __forceinline__ void task_pre(const ApplyCtx<T>& C, const Entry& e, Pre<T>& P, int* idx) {
     const int tid = threadIdx.x;
     P.gi = -1;
     P.pi = -1;
     if (e.kind == TK_GATHER) return;
-    if (e.kind == TK_UPW || e.kind == TK_DNW) {
-        taskw_pre(C.wdesc, C.sigma, C.blist, e, idx, wd);
-        return;
-    }
     if (e.kind == TK_SUBUP || e.kind == TK_SUBDN) return;
     if (e.kind == TK_HUP || e.kind == TK_HROOT || e.kind == TK_HDN) {
         if (e.b_off & 1) {                       // leaf: the rows of I^s it owns, in HSS order
@@ -715,24 +738,24 @@ __device__ __forceinline__ void task_pre(const ApplyCtx<T>& C, const Entry& e, P
     const T* F = C.front + e.base;
     switch (e.kind) {
     case TK_UPDIAG: {
-        gemv_pre(F, m, (int)m, m_i, e.a, P.v);
+        gemv_pre_task(task_rows<T>(e), F, m, (int)m, m_i, e.a, P.v);
         for (int c = tid; c < m_i; c += AT) idx[c] = C.sigma[i_off + c];
         const int r = e.a + tid;
-        if (tid < APPLY_ROWS && r < m) {
+        if (tid < task_rows<T>(e) && r < m) {
             if (r >= m_i) P.gi = C.blist[b_off + r - m_i];
             else if (e.fin) P.pi = C.perm[i_off + r];
         }
         break;
     }
     case TK_UP: {
-        gemv_pre(F + m_i, m, m_b, m_i, e.a, P.v);
+        gemv_pre_task(task_rows<T>(e), F + m_i, m, m_b, m_i, e.a, P.v);
         for (int c = tid; c < m_i; c += AT) idx[c] = C.sigma[i_off + c];
-        if (tid < APPLY_ROWS && e.a + tid < m_b) P.gi = C.blist[b_off + e.a + tid];
+        if (tid < task_rows<T>(e) && e.a + tid < m_b) P.gi = C.blist[b_off + e.a + tid];
         break;
     }
     case TK_DPART: {
         const int nc = min(e.k, m_i - e.b);
-        gemv_pre(F + (int64_t)e.b * m, m, m_i, nc, e.a, P.v);
+        gemv_pre_task(task_rows<T>(e), F + (int64_t)e.b * m, m, m_i, nc, e.a, P.v);
         for (int c = tid; c < nc; c += AT) idx[c] = C.sigma[i_off + e.b + c];
         break;
     }
@@ -740,9 +763,9 @@ __device__ __forceinline__ void task_pre(const ApplyCtx<T>& C, const Entry& e, P
         if (e.fin && e.a + tid < m_i) P.pi = C.perm[i_off + e.a + tid];
         break;
     case TK_DN: {
-        gemv_pre(F + (int64_t)m_i * m, m, m_i, m_b, e.a, P.v);
+        gemv_pre_task(task_rows<T>(e), F + (int64_t)m_i * m, m, m_i, m_b, e.a, P.v);
         for (int j = tid; j < m_b; j += AT) idx[j] = C.blist[b_off + j];
-        if (tid < APPLY_ROWS && e.a + tid < m_i) P.pi = C.perm[i_off + e.a + tid];
+        if (tid < task_rows<T>(e) && e.a + tid < m_i) P.pi = C.perm[i_off + e.a + tid];
         break;
     }
     case TK_UPDOT: case TK_DNDOT: {
@@ -795,7 +818,7 @@ __device__ __forceinline__ void task_pre(const ApplyCtx<T>& C, const Entry& e, P
 // memory use before the caller's next barrier.
 template <typename T, typename V>
 __device__ __forceinline__ void task_run(const ApplyCtx<T>& C, const Entry& e, const Pre<T>& P, const int* idx, T* vec,
-                                         T (*red)[APPLY_ROWS], const int (*wd)[8], int n, const V* __restrict__ x,
+                                         T (*red)[APPLY_ROWS], int n, const V* __restrict__ x,
                                          V* __restrict__ out, T* y, T* z, T* tup, T* tdn, T* dpart, T* us,
                                          const Sched* Sp) {
     const int tid = threadIdx.x;
@@ -818,10 +841,6 @@ __device__ __forceinline__ void task_run(const ApplyCtx<T>& C, const Entry& e, c
         return;
     }
     __syncthreads();
-    if (e.kind == TK_UPW || e.kind == TK_DNW) {
-        taskw_run<T, V>(C, e, idx, vec, wd, out, y, z);
-        return;
-    }
     if (e.kind == TK_HUP || e.kind == TK_HROOT || e.kind == TK_HDN) {
         ulv_task<T, V>(C, e, idx, vec, red, out, y, z, us);
         return;
@@ -837,9 +856,9 @@ __device__ __forceinline__ void task_run(const ApplyCtx<T>& C, const Entry& e, c
     case TK_UPDIAG: {
         for (int c = tid; c < m_i; c += AT) vec[c] = ldw(y + i_off + idx[c]);
         __syncthreads();
-        const T sum = gemv_rows64(F, m, (int)m, m_i, e.a, vec, red, P.v);
+        const T sum = gemv_task(task_rows<T>(e), F, m, (int)m, m_i, e.a, vec, red, P.v);
         const int r = e.a + tid;
-        if (tid < APPLY_ROWS && r < m) {
+        if (tid < task_rows<T>(e) && r < m) {
             if (r < m_i) {
                 stw(z + i_off + r, sum);
                 if (e.fin) out[P.pi] = to_val(sum);
@@ -852,7 +871,7 @@ __device__ __forceinline__ void task_run(const ApplyCtx<T>& C, const Entry& e, c
     case TK_UP: {
         for (int c = tid; c < m_i; c += AT) vec[c] = ldw(y + i_off + idx[c]);
         __syncthreads();
-        const T sum = gemv_rows64(F + m_i, m, m_b, m_i, e.a, vec, red, P.v);
+        const T sum = gemv_task(task_rows<T>(e), F + m_i, m, m_b, m_i, e.a, vec, red, P.v);
         if (P.gi >= 0) stw(y + P.gi, ldw(y + P.gi) - sum);
         break;
     }
@@ -860,9 +879,9 @@ __device__ __forceinline__ void task_run(const ApplyCtx<T>& C, const Entry& e, c
         const int nc = min(e.k, m_i - e.b);
         for (int c = tid; c < nc; c += AT) vec[c] = ldw(y + i_off + idx[c]);
         __syncthreads();
-        const T sum = gemv_rows64(F + (int64_t)e.b * m, m, m_i, nc, e.a, vec, red, P.v);
+        const T sum = gemv_task(task_rows<T>(e), F + (int64_t)e.b * m, m, m_i, nc, e.a, vec, red, P.v);
         const int r = e.a + tid;
-        if (tid < APPLY_ROWS && r < m_i) stw(dpart + e.aux + (int64_t)(e.b / e.k) * m_i + r, sum);
+        if (tid < task_rows<T>(e) && r < m_i) stw(dpart + e.aux + (int64_t)(e.b / e.k) * m_i + r, sum);
         break;
     }
     case TK_DSUM: {
@@ -887,9 +906,9 @@ __device__ __forceinline__ void task_run(const ApplyCtx<T>& C, const Entry& e, c
     case TK_DN: {
         for (int j = tid; j < m_b; j += AT) vec[j] = ldw(z + idx[j]);
         __syncthreads();
-        const T sum = gemv_rows64(F + (int64_t)m_i * m, m, m_i, m_b, e.a, vec, red, P.v);
+        const T sum = gemv_task(task_rows<T>(e), F + (int64_t)m_i * m, m, m_i, m_b, e.a, vec, red, P.v);
         const int r = e.a + tid;
-        if (tid < APPLY_ROWS && r < m_i) {
+        if (tid < task_rows<T>(e) && r < m_i) {
             const T v = ldw(z + i_off + r) + sum;
             stw(z + i_off + r, v);
             out[P.pi] = to_val(v);
@@ -1115,9 +1134,7 @@ __global__ void sched_deps_kernel(Sched S, const int32_t* __restrict__ node, int
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= S.nq) return;
     const Entry e = decode(S.q, t);
-    Deps d;
-    d.n = 0;
-    if (e.kind != TK_UPW && e.kind != TK_DNW) d = task_deps(S, node, e);
+    const Deps d = task_deps(S, node, e);
     int c[3] = {0, 0, 0}, need[3] = {0, 0, 0};
     for (int i = 0; i < d.n; ++i) {
         c[i] = (int)(d.c[i] - S.ctl);
@@ -1155,34 +1172,6 @@ __device__ bool wait_gather(const Sched* S) {
     return wait_geq(*S, S->ctl + 1, S->ngather, t0);
 }
 
-// Dependencies of a warp-node task, checked by warp 0: lane j < e.a waits for
-// node j's children (TK_UPW; lane 0 also for the gather) or for its parent's
-// final rows and its own diagonal rows (TK_DNW).  True on every lane when all
-// are met.
-__device__ bool wait_deps_w(const Sched& S, const int32_t* node, const int32_t* wdesc, const Entry& e) {
-    const int lane = threadIdx.x & 31;
-    bool ok = !(ld_relaxed(S.ctl + 2) || ld_relaxed(S.err));
-    const int32_t* cnt = S.ctl + CTL_WORDS;
-    const int nn = S.nn;
-    uint64_t t0 = 0;
-    if (ok && e.kind == TK_UPW && lane == 0) ok = wait_geq(S, S.ctl + 1, S.ngather, t0);
-    if (ok && lane < e.a) {
-        const int s = wdesc[(e.base + lane) * 8];
-        if (e.kind == TK_UPW) {
-            const int c0 = nf(node, s, 2), c1 = nf(node, s, 3);
-            if (c0 >= 0) ok = ok && wait_geq(S, cnt + CN_UP * nn + c0, S.need[CN_UP * nn + c0], t0);
-            if (c1 >= 0) ok = ok && wait_geq(S, cnt + CN_UP * nn + c1, S.need[CN_UP * nn + c1], t0);
-        } else {
-            const int p = nf(node, s, 1);
-            if (p >= 0) ok = ok && wait_geq(S, cnt + CN_FIN * nn + p, S.need[CN_FIN * nn + p], t0);
-            ok = ok && wait_geq(S, cnt + CN_DIAG * nn + s, S.need[CN_DIAG * nn + s], t0);
-        }
-    }
-    ok = __all_sync(0xffffffffu, ok);
-    __threadfence();
-    return ok;
-}
-
 // counters a finished task signals (bit per CN_*), -1 bit 31 for the gather count
 __device__ __forceinline__ unsigned task_signals(const Entry& e) {
     switch (e.kind) {
@@ -1216,7 +1205,6 @@ __global__ void __launch_bounds__(AT, apply_min_blocks<T>()) apply_dataflow_kern
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T red[AW][APPLY_ROWS];
     __shared__ int s_task, s_ok;
-    __shared__ int wd[AW][8];
     T* vec = reinterpret_cast<T*>(smem_raw);
     int* idx = reinterpret_cast<int*>(vec + vlen);
     int32_t* cnt = S.ctl + CTL_WORDS;
@@ -1237,39 +1225,24 @@ __global__ void __launch_bounds__(AT, apply_min_blocks<T>()) apply_dataflow_kern
         }
         const Entry e = decode(S.q, t);
         Pre<T> P;
-        task_pre(C, e, P, idx, wd);
-        const bool warp_nodes = e.kind == TK_UPW || e.kind == TK_DNW;
+        task_pre(C, e, P, idx);
         // a subtree task runs for tens of microseconds: the CTA takes its next
         // ticket when it ends, so no ready task waits behind it
         const bool long_task = e.kind == TK_SUBUP || e.kind == TK_SUBDN;
-        if (warp_nodes ? threadIdx.x < 32 : threadIdx.x == 0) {
-            const bool ok = warp_nodes ? wait_deps_w(S, C.node, C.wdesc, e) : wait_deps(S, d0, d1);
-            if (threadIdx.x == 0) {
-                s_ok = ok ? 1 : 0;
-                if (ok && !long_task) next = atomicAdd(S.ctl, 1);
-            }
+        if (threadIdx.x == 0) {
+            const bool ok = wait_deps(S, d0, d1);
+            s_ok = ok ? 1 : 0;
+            if (ok && !long_task) next = atomicAdd(S.ctl, 1);
         }
         __syncthreads();
         if (!s_ok) break;
-        task_run<T, V>(C, e, P, idx, vec, red, wd, n, x, out, y, z, tup, tdn, dpart, us, &S);
+        task_run<T, V>(C, e, P, idx, vec, red, n, x, out, y, z, tup, tdn, dpart, us, &S);
         // publish: the barrier orders every thread's stores before the
         // signalling threads' gpu-scope fences, which order them before the
         // signals
         __syncthreads();
         if (long_task && threadIdx.x == 0) next = atomicAdd(S.ctl, 1);
-        if (warp_nodes) {
-            const int lane = threadIdx.x;
-            if (lane < e.a) {
-                const int sj = wd[lane][0];
-                __threadfence();
-                if (e.kind == TK_UPW) {
-                    atomicAdd(cnt + CN_UP * S.nn + sj, 1);
-                    atomicAdd(cnt + CN_DIAG * S.nn + sj, 1);
-                } else {
-                    atomicAdd(cnt + CN_FIN * S.nn + sj, 1);
-                }
-            }
-        } else if (threadIdx.x == 0 && (e.kind == TK_HUP || e.kind == TK_HROOT || e.kind == TK_HDN)) {
+        if (threadIdx.x == 0 && (e.kind == TK_HUP || e.kind == TK_HROOT || e.kind == TK_HDN)) {
             __threadfence();
             atomicAdd(cnt + (e.kind == TK_HUP ? hu_index(S, e.s) : hd_index(S, e.s)), 1);
             if (e.kind != TK_HUP && (e.b_off & 1)) {        // a leaf wrote its rows of z(I^s)
@@ -1300,13 +1273,12 @@ __global__ void __launch_bounds__(AT, apply_min_blocks<T>()) apply_group_kernel(
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ T red[AW][APPLY_ROWS];
-    __shared__ int wd[AW][8];
     T* vec = reinterpret_cast<T*>(smem_raw);
     int* idx = reinterpret_cast<int*>(vec + vlen);
     const Entry e = decode(q, blockIdx.x);
     Pre<T> P;
-    task_pre(C, e, P, idx, wd);
-    task_run<T, V>(C, e, P, idx, vec, red, wd, n, x, out, y, z, tup, tdn, dpart, us, nullptr);
+    task_pre(C, e, P, idx);
+    task_run<T, V>(C, e, P, idx, vec, red, n, x, out, y, z, tup, tdn, dpart, us, nullptr);
 }
 
 bool levels_schedule_requested() {
@@ -1316,7 +1288,7 @@ bool levels_schedule_requested() {
 
 template <typename T>
 ApplyCtx<T> make_ctx(const FactorData& F) {
-    return ApplyCtx<T>{F.d_node, F.d_blist, F.d_sigma, F.d_perm, static_cast<const T*>(F.d_front), F.d_wdesc,
+    return ApplyCtx<T>{F.d_node, F.d_blist, F.d_sigma, F.d_perm, static_cast<const T*>(F.d_front),
                        reinterpret_cast<const UlvDev*>(F.d_ulvdev), F.d_ulv_ord, F.d_foff, F.d_sublist};
 }
 
@@ -1422,12 +1394,12 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
     std::vector<int64_t> groups{0};
     std::vector<int64_t> dpoff(std::max(nn, 1), 0);
     std::vector<int32_t> dcols(std::max(nn, 1), DIAG_COLS);   // column chunk of each node's diagonal tasks
-    auto push = [&](int kind, int s, int a, int b, bool fin) {
+    auto push = [&](int kind, int s, int a, int b, bool fin, int rows = APPLY_ROWS) {
         const bool lr = kind == TK_UPDOT || kind == TK_UPAXPY || kind == TK_DNDOT || kind == TK_DNAXPY;
         const int64_t base = kind == TK_GATHER ? 0 : lr ? (int64_t)F.lr_ptr[s] : F.foff[s];
         const int64_t aux = lr ? F.lr_toff[s] : (kind == TK_DPART || kind == TK_DSUM) ? dpoff[s] : 0;
         const bool g = kind == TK_GATHER;
-        const int32_t w[QW] = {(fin ? TK_FINAL : 0) | (kind << TK_SHIFT) | s, a, b,
+        const int32_t w[QW] = {(rows == FINE_ROWS ? TK_FINE : 0) | (fin ? TK_FINAL : 0) | (kind << TK_SHIFT) | s, a, b,
                                g ? 0 : F.m_i(s), g ? 0 : F.m_b(s), g ? 0 : F.info(s, 4), g ? 0 : F.info(s, 6),
                                lr ? F.lr_k[s] : (kind == TK_DPART || kind == TK_DSUM) ? dcols[s] : 0,
                                (int32_t)(uint32_t)(uint64_t)base, (int32_t)(uint32_t)((uint64_t)base >> 32),
@@ -1449,11 +1421,6 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
     F.dpart_total = 0;
     // low-rank dot tasks: one LR_CHUNK-row chunk times one column group
     const int dgw = (AT / 32) * (F.esize <= 8 ? 2 : 1);
-    // warp-node levels: the bottom range of levels whose nodes are all dense
-    // and tiny; a task takes up to AW consecutive nodes of one level
-    auto tiny = [&](int s) {
-        return mode(s) == 0 && F.m_i(s) <= WN_MI && F.m_i(s) + F.m_b(s) <= WN_M && F.m_b(s) <= WREG;
-    };
     // bottom subtrees: the shallowest level Ls from which every node down to
     // the leaves is dense with small fronts and every subtree fits one task
     // (NDHSS_APPLY_SUBTREES=0 keeps per-node tasks everywhere)
@@ -1474,7 +1441,7 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
             nlev[s] = 1 + std::max(c0 >= 0 ? nlev[c0] : 0, c1 >= 0 ? nlev[c1] : 0);
         }
         auto node_ok = [&](int s) {
-            return mode(s) == 0 && !ulv_node(s) && F.m_i(s) <= 2 * WN_MI && F.m_b(s) <= 4 * WREG;
+            return mode(s) == 0 && !ulv_node(s) && F.m_i(s) <= SUB_MI && F.m_b(s) <= SUB_MB;
         };
         // a subtree fits: nodes, levels, nodes and staged inputs per level, vector segment
         auto root_ok = [&](int r) {
@@ -1608,36 +1575,6 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
         }
     }
     F.sched_sub_level = Ls;
-    int L_w = F.depth + 1;
-    for (int l = std::min(F.depth, Ls - 1); l >= 0 && Ls > F.depth; --l) {
-        bool all = true;
-        for (int s : F.levels[l]) all = all && tiny(s);
-        if (!all) break;
-        L_w = l;
-    }
-    std::vector<int32_t> wdesc;
-    std::vector<int64_t> wlev(F.depth + 2, 0);      // first warp-node index of each level
-    for (int l = L_w; l <= F.depth; ++l) {
-        wlev[l] = (int64_t)wdesc.size() / 8;
-        for (int s : F.levels[l]) {
-            const uint64_t fo = (uint64_t)F.foff[s];
-            const int32_t d[8] = {s, F.m_i(s), F.m_b(s), F.info(s, 4), F.info(s, 6),
-                                  (int32_t)(uint32_t)fo, (int32_t)(uint32_t)(fo >> 32), 0};
-            wdesc.insert(wdesc.end(), d, d + 8);
-            need[CN_UP * nn + s] = 1;
-            need[CN_DIAG * nn + s] = 1;
-            need[CN_FIN * nn + s] = 1;
-        }
-    }
-    auto push_w = [&](int kind, int l) {
-        const int cnt = (int)F.levels[l].size();
-        for (int j = 0; j < cnt; j += AW) {
-            const int64_t base = wlev[l] + j;
-            const int32_t w[QW] = {(kind << TK_SHIFT) | F.levels[l][j], std::min(AW, cnt - j), l, 0, 0, 0, 0, 0,
-                                   (int32_t)(uint32_t)(uint64_t)base, (int32_t)(uint32_t)((uint64_t)base >> 32), 0, 0};
-            q.insert(q.end(), w, w + QW);
-        }
-    };
     auto ulv_front = [&](int s) { return !F.ulv_root_of.empty() && F.ulv_root_of[s] >= 0; };
     const int ng = ceil_div(F.n, GATHER_CHUNK);
     for (int i = 0; i < ng; ++i) push(TK_GATHER, 0, i * GATHER_CHUNK, GATHER_CHUNK, false);
@@ -1654,15 +1591,35 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
         }
         cut();
     }
-    for (int l = F.depth; l >= L_w; --l) {
-        push_w(TK_UPW, l);
-        cut();
-    }
     // The diagonal step of the nodes not fused into their up-sweep tasks:
     // column-chunk partial products, then their sums.  Same dependencies as
     // the node's up-sweep, so they are queued with it: ready together, and the
     // tickets of the up-sweep chain above do not hold them back.
-    const int l_top = std::min({F.depth, L_w - 1, Ls - 1});
+    const int l_top = std::min(F.depth, Ls - 1);
+    // Rows per row task.  FP64 levels with fewer 64-row tasks than FINE_TASKS
+    // (four per SM) take FINE_ROWS: their time is the FP64 pipe's, so it is the
+    // number of SMs with work that counts (one apply, 256 x 256 P2 Helmholtz,
+    // dense complex128, 1.45 GB: 1571 us with 64 rows everywhere, 1005 so; all
+    // levels fine is 1079).
+    constexpr int FINE_TASKS = 4 * 152;
+    auto pick_rows = [&](int64_t tasks) { return F.prec == NDHSS_FP64 && tasks < FINE_TASKS ? FINE_ROWS : APPLY_ROWS; };
+    std::vector<int> rows_up(F.depth + 1, APPLY_ROWS), rows_dn(F.depth + 1, APPLY_ROWS);
+    for (int l = 0; l <= l_top; ++l) {
+        int64_t up = 0, dn = 0;
+        for (int s : F.levels[l]) {
+            const int mi = F.m_i(s), mb = F.m_b(s);
+            if (mi == 0) continue;
+            if (fused(s)) {
+                up += ceil_div(mi + mb, APPLY_ROWS);
+            } else {
+                if (!ulv_front(s)) up += (int64_t)ceil_div(mi, DIAG_COLS) * ceil_div(mi, APPLY_ROWS);
+                if (mode(s) == 0) up += ceil_div(mb, APPLY_ROWS);
+            }
+            if (mode(s) == 0) dn += ceil_div(mi, APPLY_ROWS);
+        }
+        rows_up[l] = pick_rows(up);
+        rows_dn[l] = pick_rows(dn);
+    }
     auto push_dpart = [&](int l) {
         for (int s : F.levels[l]) {
             const int mi = F.m_i(s);
@@ -1674,8 +1631,8 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
             dpoff[s] = F.dpart_total;
             F.dpart_total += (int64_t)nch * mi;
             for (int c0 = 0; c0 < mi; c0 += dcols[s])
-                for (int r0 = 0; r0 < mi; r0 += APPLY_ROWS) push(TK_DPART, s, r0, c0, false);
-            need[CN_DPART * nn + s] = nch * ceil_div(mi, APPLY_ROWS);
+                for (int r0 = 0; r0 < mi; r0 += rows_up[l]) push(TK_DPART, s, r0, c0, false, rows_up[l]);
+            need[CN_DPART * nn + s] = nch * ceil_div(mi, rows_up[l]);
         }
     };
     auto push_dsum = [&](int l) {
@@ -1692,14 +1649,14 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
         for (int s : F.levels[l]) {
             const int mi = F.m_i(s), mb = F.m_b(s);
             if (fused(s)) {
-                const int rows = mi + mb, cnt = ceil_div(rows, APPLY_ROWS);
-                for (int r0 = 0; r0 < rows; r0 += APPLY_ROWS) push(TK_UPDIAG, s, r0, 0, diag_final(s));
+                const int rows = mi + mb, cnt = ceil_div(rows, rows_up[l]);
+                for (int r0 = 0; r0 < rows; r0 += rows_up[l]) push(TK_UPDIAG, s, r0, 0, diag_final(s), rows_up[l]);
                 need[CN_UP * nn + s] = cnt;
                 need[CN_DIAG * nn + s] = cnt;
                 if (diag_final(s)) need[CN_FIN * nn + s] = cnt;
             } else if (mi > 0 && mb > 0 && mode(s) == 0) {
-                for (int j0 = 0; j0 < mb; j0 += APPLY_ROWS) push(TK_UP, s, j0, 0, false);
-                need[CN_UP * nn + s] = ceil_div(mb, APPLY_ROWS);
+                for (int j0 = 0; j0 < mb; j0 += rows_up[l]) push(TK_UP, s, j0, 0, false, rows_up[l]);
+                need[CN_UP * nn + s] = ceil_div(mb, rows_up[l]);
             } else if (mi > 0 && mb > 0 && mode(s) == 1) {
                 for (int r0 = 0; r0 < mi; r0 += LR_CHUNK)
                     for (int a0 = 0; a0 < F.lr_k[s]; a0 += dgw) push(TK_UPDOT, s, r0, a0, false);
@@ -1769,7 +1726,7 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
             if (F.ulv_recs[i].level == lv) push_u(TK_HDN, i);
         cut();
     }
-    for (int l = 0; l < std::min(L_w, Ls); ++l) {
+    for (int l = 0; l <= l_top; ++l) {
         for (int s : F.levels[l]) {
             if (F.m_i(s) == 0 || diag_final(s) || mode(s) != 1) continue;
             for (int r0 = 0; r0 < F.m_b(s); r0 += LR_CHUNK)
@@ -1784,17 +1741,11 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
                 continue;
             }
             if (diag_final(s)) continue;
-            if (mode(s) == 0) {
-                for (int i0 = 0; i0 < F.m_i(s); i0 += APPLY_ROWS) push(TK_DN, s, i0, 0, true);
-            } else {
-                for (int r0 = 0; r0 < F.m_i(s); r0 += APPLY_ROWS) push(TK_DNAXPY, s, r0, 0, true);
-            }
-            need[CN_FIN * nn + s] = ceil_div(F.m_i(s), APPLY_ROWS);
+            const bool dense = mode(s) == 0;
+            const int rows = dense ? rows_dn[l] : APPLY_ROWS;
+            for (int r0 = 0; r0 < F.m_i(s); r0 += rows) push(dense ? TK_DN : TK_DNAXPY, s, r0, 0, true, rows);
+            need[CN_FIN * nn + s] = ceil_div(F.m_i(s), rows);
         }
-        cut();
-    }
-    for (int l = L_w; l <= F.depth; ++l) {
-        push_w(TK_DNW, l);
         cut();
     }
     if (Ls <= F.depth) {
@@ -1805,8 +1756,6 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
     F.sched_ngather = ng;
     F.sched_groups = groups;
     F.sched_vlen = std::max(F.sched_vlen, std::max(std::max(F.max_mi, F.max_mb), LR_CHUNK));
-    if (L_w <= F.depth) F.sched_vlen = std::max(F.sched_vlen, AW * WREG);
-    F.sched_warp_level = L_w;
     if (F.sched_n >= (int64_t)INT32_MAX / QW) return set_error(NDHSS_ERR_INVALID_ARG, "apply: task queue too long");
     ndhss_status rc = NDHSS_OK;
     auto up = [&](auto** dst, const auto& v) {
@@ -1822,7 +1771,6 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
     };
     up(&F.d_sched, q);
     up(&F.d_need, need);
-    up(&F.d_wdesc, wdesc);
     up(&F.d_sublist, sublist);
     if (nrec) {
         if (pool_malloc_async(&F.d_ulvdev, udev.size() * sizeof(UlvDev), st) != cudaSuccess ||

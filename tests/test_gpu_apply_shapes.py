@@ -33,7 +33,7 @@ def _rand(shape, cplx, seed):
 
 @pytest.mark.parametrize("nrhs", [1, 4, 5, 31, 32])
 @pytest.mark.parametrize("kind,N,leaf", [("poisson", 4, 64), ("poisson", 41, 16), ("helmholtz", 3, 64),
-                                         ("helmholtz", 29, 24)])
+                                         ("helmholtz", 29, 24), ("helmholtz", 52, 16)])
 def test_fp64_multi_apply_matches_single_applies(nd, kind, N, leaf, nrhs):
     P = poisson_dirichlet(N, seed=1) if kind == "poisson" else helmholtz_impedance(N, 2, 6.0, seed=1)
     tree = nd.ndhss_build_tree(P.coords, P.A.indptr, P.A.indices, leaf)
