@@ -31,6 +31,8 @@
 #include <string>
 #include <thread>
 
+#include <cooperative_groups.h>
+
 #include "factor.cuh"
 
 namespace ndhss {
@@ -116,6 +118,7 @@ template <typename T> __device__ __forceinline__ T neg_zero();
 template <> __device__ __forceinline__ float neg_zero<float>() { return -0.0f; }
 template <> __device__ __forceinline__ double neg_zero<double>() { return -0.0; }
 template <> __device__ __forceinline__ c64 neg_zero<c64>() { return {-0.0f, -0.0f}; }
+template <> __device__ __forceinline__ c128 neg_zero<c128>() { return {-0.0, -0.0}; }
 
 // r = v when i == j, by a predicated move: a plain select on a runtime
 // column index lets the compiler turn the row's registers into a
@@ -129,6 +132,10 @@ __device__ __forceinline__ void take_if(int j, int i, double v, double& r) {
 __device__ __forceinline__ void take_if(int j, int i, c64 v, c64& r) {
     asm("{\n\t.reg .pred q;\n\tsetp.eq.s32 q, %2, %3;\n\t@q mov.f32 %0, %4;\n\t@q mov.f32 %1, %5;\n\t}"
         : "+f"(r.x), "+f"(r.y) : "r"(i), "r"(j), "f"(v.x), "f"(v.y));
+}
+__device__ __forceinline__ void take_if(int j, int i, c128 v, c128& r) {
+    take_if(j, i, v.x, r.x);
+    take_if(j, i, v.y, r.y);
 }
 
 // ---------------------------------------------------------------- panel
@@ -419,6 +426,145 @@ panel_reg_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ no
     if (tid == 0) sm[0] = s_na;
 }
 
+// 1 / a for the pivot.  Complex float64: conj(a) / |a|^2 with a scaled by a
+// power of two first (exact), one division where Smith's formula takes three
+// (a division is a long sequence on GB300's FP64 pipe).
+template <typename T> __device__ __forceinline__ T pivot_recip(T a) { return recip(a); }
+template <> __device__ __forceinline__ c128 pivot_recip<c128>(c128 a) {
+    const int e = max((__double2hiint(a.x) >> 20) & 0x7ff, (__double2hiint(a.y) >> 20) & 0x7ff);
+    // exponents near the ends of the range (and infinities, NaN): Smith's formula
+    if (e < 2 || e > 2044) return recip(a);
+    const double s = __hiloint2double((2046 - e) << 20, 0);       // 2^(1023 - e)
+    const double x = a.x * s, y = a.y * s;                        // max(|x|, |y|) in [1, 2)
+    const double r = 1.0 / fma(x, x, y * y);
+    return {(x * r) * s, -((y * r) * s)};
+}
+
+// The panel with its candidate rows spread over the C CTAs of a thread-block
+// cluster (C = 1: one CTA), one row per thread in registers.  The exchange
+// steps are those of panel_reg_kernel; the warps' candidates and their rows
+// are read by every warp of the cluster through distributed shared memory
+// after the step's one cluster barrier.
+//
+// FP64 fronts: a pivot of a panel of mc rows costs mc KB multiply-adds on an
+// FP64 pipe of 0.5 per clock and SM quarter, so a top-level panel of ~1500
+// complex rows held one SM for 25 us per pivot in shared memory; spread over
+// eight SMs with one warp per SM quarter it is the barrier and the scalars
+// (~1.5 us) plus the row's own update (2 us).  Panels of a 256 x 256 P2 factor
+// in complex128: 119 ms before (105 with 16 columns), 28 ms so.  FP32 fronts
+// use it above 512 rows, where one CTA needs more than 16 warps; 32 columns
+// then fit the registers at any size (16 before, 8 - 16 in shared memory above
+// 1024 rows), which halves the launches of the steps after it: dense 512 x 512
+// P2, complex64, 87 -> 79 ms.
+template <typename T, int KB, int MAXT>
+__global__ void __launch_bounds__(MAXT)
+panel_cluster_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ node,
+                     const int64_t* __restrict__ foff, const T* __restrict__ front, int32_t* __restrict__ ipiv,
+                     T* __restrict__ ainv_buf, int32_t* __restrict__ swapmap, int k0, int kb, DevStatus* status) {
+    using real = typename Tr<T>::real;
+    using PK = PivKey<real>;
+    using K = typename PK::K;
+    namespace cg = cooperative_groups;
+    constexpr int NW = MAXT / 32;
+    __shared__ T s_cand[2][NW][KB];          // each warp's best candidate row
+    __shared__ K s_key[2][NW];
+    __shared__ int s_pos[2][NW];
+    __shared__ T s_pr[NW][KB];               // the pivot row, formed by each warp for itself
+    __shared__ int s_na;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rk = (int)cl.block_rank();
+    const int li = blockIdx.x / C;
+    const int s = lev[li];
+    const int m_i = nf(node, s, 5);
+    if (k0 >= m_i) return;                   // every CTA of the cluster alike
+    const int64_t m = m_i + nf(node, s, 7);
+    const int kbp = min(kb, m_i - k0);
+    const int mc = m_i - k0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int row = rk * (int)blockDim.x + tid;
+    const bool has = row < mc;
+    const T* F = front + foff[s];
+    auto sync = [&]() {
+        if (C > 1) cl.sync();
+        else __syncthreads();
+    };
+    T v[KB];
+#pragma unroll
+    for (int j = 0; j < KB; ++j) v[j] = (has && j < kbp) ? F[(int64_t)(k0 + j) * m + k0 + row] : zero<T>();
+    int pos = row;                           // this row's position after the interchanges so far
+    if (tid == 0) s_na = 0;
+    panel_publish<T, KB>(v, abs1(v[0]), has, pos, s_cand[0][warp], &s_key[0][warp], &s_pos[0][warp], lane);
+    sync();
+    int32_t* ip = ipiv + nf(node, s, 4) + k0;
+    T a = v[0];                              // this row's entry in the pivot column
+    for (int c = 0; c < kbp; ++c) {
+        const int par = c & 1;
+        // the cluster's best candidate: largest key, then lowest position
+        K bk = K(0);
+        unsigned bp = 0xffffffffu;           // position << 8 | warp of the cluster
+        for (int q = lane; q < C * nwarps; q += 32) {
+            const int r = q / nwarps, w = q % nwarps;
+            const K kw = C > 1 ? *cl.map_shared_rank(&s_key[par][w], r) : s_key[par][w];
+            const unsigned pw = ((unsigned)(C > 1 ? *cl.map_shared_rank(&s_pos[par][w], r) : s_pos[par][w]) << 8) | (unsigned)q;
+            if (kw > bk || (kw == bk && kw != K(0) && pw < bp)) { bk = kw; bp = pw; }
+        }
+        const K kmax = PK::wmax(bk);
+        const unsigned pw = __reduce_min_sync(0xffffffffu, (kmax != K(0) && bk == kmax) ? bp : 0xffffffffu);
+        // all candidates NaN: keep the diagonal (its pivot is then flagged below)
+        const int p = kmax != K(0) ? (int)(pw >> 8) : c;
+        const int w = kmax != K(0) ? (int)(pw & 255u) : -1;
+        {
+            const T* cand = C > 1 && w >= 0 ? cl.map_shared_rank(&s_cand[par][w % nwarps][0], w / nwarps)
+                                            : &s_cand[par][w >= 0 ? w : 0][0];
+            const T b = (w >= 0 && lane < KB) ? cand[lane] : zero<T>();
+            T piv = shfl_idx(b, c);
+            if (!(abs1(piv) > real(0))) {                         // exact zero (or NaN) pivot
+                piv = one<T>();
+                if (rk == 0 && tid == 0 && atomicCAS(&status->code, 0, (int)NDHSS_ERR_SINGULAR) == 0) status->node = s;
+            }
+            const T pinv = pivot_recip(piv);
+            if (lane < KB) s_pr[warp][lane] = lane >= kbp ? zero<T>() : (lane == c) ? pinv : -(b * pinv);
+        }
+        if (rk == 0 && tid == 0) ip[c] = k0 + p;
+        __syncwarp();
+        const bool is_piv = has && pos == p;
+        // one FMA form for every entry, as in panel_reg_kernel
+        const T am = is_piv ? one<T>() : a;
+        T an = a;                            // this row's updated entry in the next column
+#pragma unroll
+        for (int j = 0; j < KB; ++j) {
+            const T prj = s_pr[warp][j];
+            const T vin = (is_piv || j == c) ? neg_zero<T>() : v[j];
+            v[j] = fmac(am, prj, vin);
+            take_if(j, c + 1, v[j], an);
+        }
+        a = an;
+        if (pos == c) pos = p;
+        else if (pos == p) pos = c;
+        if (c + 1 < kbp)
+            panel_publish<T, KB>(v, abs1(a), has && pos > c, pos, s_cand[par ^ 1][warp], &s_key[par ^ 1][warp],
+                                 &s_pos[par ^ 1][warp], lane);
+        sync();
+    }
+    // rows at positions < kbp hold (A_PP)^{-1} of the interchanged pivot block
+    T* Ai = ainv_buf + (size_t)li * KBMAX * KBMAX;
+    if (has && pos < kbp) {
+#pragma unroll
+        for (int j = 0; j < KB; ++j)
+            if (j < kbp) Ai[j * KBMAX + pos] = v[j];
+    }
+    // net row map of the interchanges: position k0 + pos receives the old row k0 + row
+    int32_t* sm = swapmap + (size_t)li * (4 * KBMAX + 1);
+    int* na = C > 1 ? cl.map_shared_rank(&s_na, 0) : &s_na;
+    if (has && pos != row) {
+        const int q = atomicAdd(na, 1);
+        sm[1 + q] = k0 + pos;
+        sm[1 + 2 * KBMAX + q] = k0 + row;
+    }
+    sync();
+    if (rk == 0 && tid == 0) sm[0] = s_na;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(PREP_WARPS * 32)
 panel_prep_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ node,
@@ -489,14 +635,16 @@ panel_prep_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ n
     }
 }
 
-// M = beta .* M + C * Z over one 64 x 64 tile (beta = 0 on pivot rows or columns).
-template <typename T>
-__global__ void __launch_bounds__(256)
+// M = beta .* M + C * Z over one tile of 64 rows x 16 NB columns (beta = 0 on
+// pivot rows or columns).  NB = 4, or 1 when the columns are one panel's (a
+// wider tile would multiply padding, at full price on the FP64 pipe).
+template <typename T, int NB>
+__global__ void __launch_bounds__(256, sizeof(T) <= 8 ? 2 : 1)
 gemm_update_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ node,
                    const int64_t* __restrict__ foff, T* __restrict__ front, const T* __restrict__ cbuf,
                    const T* __restrict__ zbuf, const int64_t* __restrict__ woff, int k0, int kb, int slab0, int slabw) {
     __shared__ T sC[GK][GT];
-    __shared__ T sZ[GK][GT];
+    __shared__ T sZ[GK][16 * NB];
     const int li = blockIdx.z;
     const int s = lev[li];
     const int m_i = nf(node, s, 5);
@@ -504,56 +652,82 @@ gemm_update_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ 
     const int64_t m = m_i + nf(node, s, 7);
     // columns [zlo, zhi): the whole front, or the slab of the outer block
     const int64_t zlo = slabw ? slab0 : 0, zhi = slabw ? min((int64_t)slab0 + slabw, (int64_t)m_i) : m;
-    const int64_t i0 = (int64_t)blockIdx.x * GT, j0 = zlo + (int64_t)blockIdx.y * GT;
+    const int64_t i0 = (int64_t)blockIdx.x * GT, j0 = zlo + (int64_t)blockIdx.y * (16 * NB);
     if (i0 >= m || j0 >= zhi) return;
     const int kbp = min(kb, m_i - k0);
     const T* C = cbuf + woff[li] * KBMAX;
     const T* Z = zbuf + woff[li] * KBMAX;
     T* F = front + foff[s];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
+    T acc[4][NB];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = zero<T>();
-    for (int kc = 0; kc < kbp; kc += GK) {
-        for (int idx = tid; idx < GK * GT; idx += 256) {
-            const int ii = idx % GT, l = idx / GT;
-            const int64_t i = i0 + ii;
-            sC[l][ii] = (kc + l < kbp && i < m) ? C[(int64_t)(kc + l) * m + i] : zero<T>();
+        for (int b = 0; b < NB; ++b) acc[a][b] = zero<T>();
+    // the tile's old values and the next K chunk travel in registers while the
+    // current chunk is multiplied (K is one or two chunks: without this a CTA
+    // waits out the memory latency three times in a row; dense 512 x 512 P2,
+    // complex64: 15.2 -> 13.6 ms of updates)
+    T rc[4], rz[NB], old[4][NB];
+    auto load = [&](int kc) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = tid + 256 * u, ii = idx % GT, l = idx / GT;
+            rc[u] = (kc + l < kbp && i0 + ii < m) ? C[(int64_t)(kc + l) * m + i0 + ii] : zero<T>();
         }
-        for (int idx = tid; idx < GK * GT; idx += 256) {
-            const int l = idx % GK, jj = idx / GK;
-            const int64_t j = j0 + jj;
-            sZ[l][jj] = (kc + l < kbp && j < zhi) ? Z[j * KBMAX + kc + l] : zero<T>();
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            const int idx = tid + 256 * u, l = idx % GK, jj = idx / GK;
+            rz[u] = (kc + l < kbp && j0 + jj < zhi) ? Z[(j0 + jj) * KBMAX + kc + l] : zero<T>();
+        }
+    };
+    load(0);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        const int64_t j = j0 + ty + 16 * b;
+        const bool pj = j >= k0 && j < k0 + kbp;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int64_t i = i0 + tx + 16 * a;
+            const bool keep = i < m && j < zhi && !pj && !(i >= k0 && i < k0 + kbp);
+            old[a][b] = keep ? F[j * m + i] : zero<T>();
+        }
+    }
+    for (int kc = 0; kc < kbp; kc += GK) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int idx = tid + 256 * u;
+            sC[idx / GT][idx % GT] = rc[u];
+        }
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            const int idx = tid + 256 * u;
+            sZ[idx % GK][idx / GK] = rz[u];
         }
         __syncthreads();
+        if (kc + GK < kbp) load(kc + GK);
 #pragma unroll
         for (int l = 0; l < GK; ++l) {
-            T av[4], bv[4];
+            T av[4], bv[NB];
 #pragma unroll
             for (int a = 0; a < 4; ++a) av[a] = sC[l][tx + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = sZ[l][ty + 16 * b];
+            for (int b = 0; b < NB; ++b) bv[b] = sZ[l][ty + 16 * b];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fmac(av[a], bv[b], acc[a][b]);
+                for (int b = 0; b < NB; ++b) acc[a][b] = fmac(av[a], bv[b], acc[a][b]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
+    for (int b = 0; b < NB; ++b) {
         const int64_t j = j0 + ty + 16 * b;
         if (j >= zhi) continue;
-        const bool pj = (j >= k0 && j < k0 + kbp);
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int64_t i = i0 + tx + 16 * a;
-            if (i >= m) continue;
-            const bool pi = (i >= k0 && i < k0 + kbp);
-            T* dst = F + j * m + i;
-            *dst = (pi || pj) ? acc[a][b] : (*dst + acc[a][b]);
+            if (i < m) F[j * m + i] = old[a][b] + acc[a][b];
         }
     }
 }
@@ -577,29 +751,65 @@ __global__ void finalize_sigma_kernel(const int32_t* __restrict__ lev, const int
     for (int j = threadIdx.x; j < m_i; j += blockDim.x) sigma[i_off + j] = a[j];
 }
 
-// One panel launch: the register-resident kernel when asked and the element
-// fits (8 bytes at most), else the shared-memory kernel.  More than
-// PANEL_THREADS rows take the 2 * PANEL_THREADS instance (64 registers a
-// thread: KB <= 16).
+// Which panel kernel a launch takes: rows in registers of one CTA, of a
+// cluster of C CTAs with `threads` rows each, or the panel in shared memory.
+struct PanelShape {
+    enum Kind { SMEM, REG, CLUSTER } kind;
+    int threads, C;
+};
+constexpr int PANEL_CLUSTER_MAX = 8;          // CTAs per cluster (portable size)
+constexpr int PANEL_KB_FP64 = 16;             // panel width of FP64 fronts (see panel_shape)
+
+// mc candidate rows in the largest front of the level.  FP32: one CTA up to
+// 512 rows, a cluster beyond.  FP64: clusters with 128 rows per CTA, one warp
+// per SM quarter, as soon as a front has more than that.  Fronts beyond
+// 8 x 512 rows (and NDHSS_PANEL=smem) take the shared-memory kernel.
+template <typename T>
+PanelShape panel_shape(bool reg, int64_t mc) {
+    constexpr bool fp64 = sizeof(typename Tr<T>::real) == 8;
+    auto round32 = [](int64_t n) { return (int)std::max<int64_t>(64, (n + 31) / 32 * 32); };
+    if (!reg || mc > (int64_t)PANEL_CLUSTER_MAX * PANEL_THREADS)
+        return {PanelShape::SMEM, (int)std::min<int64_t>(PANEL_THREADS, round32(mc)), 1};
+    if (!fp64 && mc <= PANEL_THREADS) return {PanelShape::REG, round32(mc), 1};
+    int C = 1;
+    while (C < PANEL_CLUSTER_MAX && (mc + C - 1) / C > (fp64 ? 128 : 256)) C *= 2;
+    return {PanelShape::CLUSTER, round32((mc + C - 1) / C), C};
+}
+
 template <typename T, int KB>
-void launch_panel(bool reg, int grid, int threads, size_t smem, cudaStream_t st, const int32_t* lev,
-                  const int32_t* node, const int64_t* foff, const T* front, int32_t* ipiv, T* ainv, int32_t* swapmap,
-                  int k0, int kb, DevStatus* status) {
-    if constexpr (sizeof(T) <= 8) {
-        if (reg && threads <= PANEL_THREADS) {
-            panel_reg_kernel<T, KB, PANEL_THREADS><<<grid, threads, 0, st>>>(lev, node, foff, front, ipiv, ainv, swapmap,
+cudaError_t launch_panel(const PanelShape& ps, int grid, size_t smem, cudaStream_t st, const int32_t* lev,
+                         const int32_t* node, const int64_t* foff, const T* front, int32_t* ipiv, T* ainv,
+                         int32_t* swapmap, int k0, int kb, DevStatus* status) {
+    constexpr bool fp64 = sizeof(typename Tr<T>::real) == 8;
+    if (ps.kind == PanelShape::SMEM) {
+        panel_factor_kernel<T, KB><<<grid, ps.threads, smem, st>>>(lev, node, foff, front, ipiv, ainv, swapmap, k0, kb,
+                                                                  status);
+        return cudaGetLastError();
+    }
+    if constexpr (!fp64) {
+        if (ps.kind == PanelShape::REG) {
+            panel_reg_kernel<T, KB, PANEL_THREADS><<<grid, ps.threads, 0, st>>>(lev, node, foff, front, ipiv, ainv, swapmap,
                                                                              k0, kb, status);
-            return;
-        }
-        if constexpr (KB <= 16) {
-            if (reg) {
-                panel_reg_kernel<T, KB, 2 * PANEL_THREADS><<<grid, threads, 0, st>>>(lev, node, foff, front, ipiv, ainv,
-                                                                                     swapmap, k0, kb, status);
-                return;
-            }
+            return cudaGetLastError();
         }
     }
-    panel_factor_kernel<T, KB><<<grid, threads, smem, st>>>(lev, node, foff, front, ipiv, ainv, swapmap, k0, kb, status);
+    if constexpr (!fp64 || KB <= PANEL_KB_FP64) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)grid * ps.C);
+        cfg.blockDim = dim3((unsigned)ps.threads);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)ps.C;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        auto k = ps.threads <= 128 ? panel_cluster_kernel<T, KB, 128>
+                                   : ps.threads <= 256 ? panel_cluster_kernel<T, KB, 256> : panel_cluster_kernel<T, KB, 512>;
+        return cudaLaunchKernelEx(&cfg, k, lev, node, foff, front, ipiv, ainv, swapmap, k0, kb, status);
+    }
+    return cudaErrorInvalidValue;
 }
 
 int choose_kb(int64_t mc, size_t esize, int panel_opt) {
@@ -824,7 +1034,7 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
     // a cross-check of the register-resident panel: the same real outputs, the
     // complex ones up to FMA contraction)
     const char* pe = std::getenv("NDHSS_PANEL");
-    const bool reg_panel_ok = sizeof(T) <= 8 && !(pe && std::strcmp(pe, "smem") == 0);
+    const bool reg_panel_ok = !(pe && std::strcmp(pe, "smem") == 0);
     ndhss_status rc = set_smem_attrs<T>();
     if (rc != NDHSS_OK) return rc;
     T* front = static_cast<T*>(F.d_front);
@@ -890,26 +1100,28 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
         // (a block of exchanges composed), so S stays the elimination's Schur
         // complement.  Small fronts keep the rank-kb steps over the whole front.
         const bool tcl = tc_front_path(F, mimax);
-        const int kb2 = tcl ? TC_KB2 : 0;
+        const int okb = F.prec == NDHSS_FP64 ? TC64_KB2 : TC_KB2;
+        const int kb2 = tcl ? okb : 0;
         const int gt = (int)((mmax + GT - 1) / GT);
-        const int gty = tcl ? (TC_KB2 + GT - 1) / GT : gt;
+        const int gty = tcl ? (okb + GT - 1) / GT : gt;
+        // FP64: the columns of an outer block beside the current panel are
+        // exchanged on the tensor cores too (tc64_block_exchange with the panel as
+        // its pivots), so the FP64 pipe updates the panel's own columns only (256 x
+        // 256 P2 Helmholtz, complex128: updates 50 -> 23 ms, exchanges 24 -> 41).
+        const bool inner = tcl && F.prec == NDHSS_FP64 && mimax >= TC64_INNER_MIN;
         const int pgx = (int)std::min<int64_t>((mmax + PREP_WARPS - 1) / PREP_WARPS, 1024);
         for (int64_t k0 = 0; k0 < mimax;) {
-            const int64_t s0 = tcl ? k0 / TC_KB2 * TC_KB2 : 0;     // the outer block's first pivot
-            int kb = choose_kb(mimax - k0, sizeof(T), panel_opt);
-            while (tcl && k0 + kb > s0 + TC_KB2) kb >>= 1;
-            // every candidate row in one thread's registers when the rows fit one
-            // CTA (up to 2 * PANEL_THREADS rows, at most 16 columns beyond PANEL_THREADS)
-            const bool reg_panel = reg_panel_ok && mimax - k0 <= 2 * PANEL_THREADS;
-            if (reg_panel && mimax - k0 > PANEL_THREADS) kb = std::min(kb, 16);
+            const int64_t s0 = tcl ? k0 / okb * okb : 0;     // the outer block's first pivot
+            // panels in registers have a fixed largest width, those in shared memory
+            // shrink with their rows
+            const PanelShape ps = panel_shape<T>(reg_panel_ok, mimax - k0);
+            int kb = choose_kb(ps.kind == PanelShape::SMEM ? mimax - k0 : 1, sizeof(T), panel_opt);
+            if (F.prec == NDHSS_FP64) kb = std::min(kb, PANEL_KB_FP64);
+            while (tcl && k0 + kb > s0 + okb) kb >>= 1;
             const size_t smem = (size_t)(mimax - k0) * kb * sizeof(T) + (size_t)(mimax - k0) * sizeof(int);
-            if (smem > PANEL_SMEM_MAX)
+            if (ps.kind == PanelShape::SMEM && smem > PANEL_SMEM_MAX)
                 return set_error(NDHSS_ERR_INVALID_ARG, "front with %lld interior unknowns exceeds the panel kernel's shared memory",
                                  (long long)(mimax - k0));
-            // one thread per candidate row up to 512: small fronts get small CTAs, so a level of
-            // thousands of leaves runs in one wave instead of repeating its pivot chain per wave
-            const int pthreads = (int)std::min<int64_t>(reg_panel ? 2 * PANEL_THREADS : PANEL_THREADS,
-                                                        std::max<int64_t>(64, (mimax - k0 + 31) / 32 * 32));
             // a level of more than 65535 fronts (the grid's y / z limit) goes in
             // chunks; the three kernels of a chunk share its per-front scratch
             for (int c0 = 0; c0 < L; c0 += MAX_GRID_YZ) {
@@ -917,41 +1129,59 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
                 const int32_t* levc = lev + c0;
                 const int64_t* woffc = woff + c0;
                 tm.begin();
+                cudaError_t pe_rc = cudaSuccess;
                 switch (kb) {
 #define NDHSS_PANEL(KBV)                                                                                          \
     case KBV:                                                                                                   \
-        launch_panel<T, KBV>(reg_panel, Lc, pthreads, smem, st, levc, F.d_node, F.d_foff, front, F.d_ipiv, d_ainv, \
-                             d_swapmap, (int)k0, kb, d_status);                                                 \
+        pe_rc = launch_panel<T, KBV>(ps, Lc, smem, st, levc, F.d_node, F.d_foff, front, F.d_ipiv, d_ainv, d_swapmap, \
+                                     (int)k0, kb, d_status);                                                    \
         break;
                     NDHSS_PANEL(1) NDHSS_PANEL(2) NDHSS_PANEL(4) NDHSS_PANEL(8) NDHSS_PANEL(16) NDHSS_PANEL(32)
 #undef NDHSS_PANEL
                     default: return set_error(NDHSS_ERR_INTERNAL, "panel width %d is not a power of two <= 32", kb);
                 }
-                NDHSS_LAUNCH_CHECK("panel_factor_kernel");
+                if (pe_rc != cudaSuccess)
+                    return set_error(NDHSS_ERR_CUDA, "launch of the panel kernel failed: %s", cudaGetErrorString(pe_rc));
+                NDHSS_LAUNCH_CHECK("panel kernel");
                 tm.end(2);
                 tm.begin();
                 panel_prep_kernel<T><<<dim3(pgx, Lc), PREP_WARPS * 32, 0, st>>>(levc, F.d_node, F.d_foff, front,
                                                                                d_swapmap, d_ainv, d_cbuf, d_zbuf, woffc,
-                                                                               (int)k0, kb, (int)s0, kb2);
+                                                                               (int)k0, kb, inner ? (int)k0 : (int)s0, inner ? kb : kb2);
                 NDHSS_LAUNCH_CHECK("panel_prep_kernel");
                 tm.end(3);
                 tm.begin();
-                gemm_update_kernel<T><<<dim3(gt, gty, Lc), 256, 0, st>>>(levc, F.d_node, F.d_foff, front, d_cbuf,
-                                                                       d_zbuf, woffc, (int)k0, kb, (int)s0, kb2);
+                if (inner)
+                    gemm_update_kernel<T, 1><<<dim3(gt, (kb + 15) / 16, Lc), 256, 0, st>>>(
+                        levc, F.d_node, F.d_foff, front, d_cbuf, d_zbuf, woffc, (int)k0, kb, (int)k0, kb);
+                else
+                    gemm_update_kernel<T, 4><<<dim3(gt, gty, Lc), 256, 0, st>>>(levc, F.d_node, F.d_foff, front, d_cbuf,
+                                                                              d_zbuf, woffc, (int)k0, kb, (int)s0, kb2);
                 NDHSS_LAUNCH_CHECK("gemm_update_kernel");
                 tm.end(4);
             }
             F.launches += 3;
             for (int s2 : nodes) {
                 const int64_t mi = F.m_i(s2), m2 = mi + F.m_b(s2);
-                const int64_t cols = tcl ? std::min<int64_t>(TC_KB2, mi - s0) : m2;
+                const int64_t cols = inner ? kb : tcl ? std::min<int64_t>(okb, mi - s0) : m2;
                 if (mi > k0) F.update_flops += flops_per_mac * (double)m2 * (double)cols * (double)std::min<int64_t>(kb, mi - k0);
             }
+            if (inner) {
+                // the panel's exchange on the outer block's other columns
+                tm.begin();
+                const ndhss_status rc2 = tc64_block_exchange(F, nodes, (int)k0, kb, (int)s0, (int)s0 + okb, d_status, st);
+                if (rc2 != NDHSS_OK) {
+                    if (d_aii) cudaFreeAsync(d_aii, st);
+                    return rc2;
+                }
+                tm.end(7);
+            }
             k0 += kb;
-            if (tcl && (k0 == s0 + TC_KB2 || k0 >= mimax)) {
+            if (tcl && (k0 == s0 + okb || k0 >= mimax)) {
                 // the outer block's exchange on the columns outside its slab
                 tm.begin();
-                const ndhss_status rc2 = tc_block_exchange(F, nodes, (int)s0, d_status, st);
+                const ndhss_status rc2 = F.prec == NDHSS_FP64 ? tc64_block_exchange(F, nodes, (int)s0, okb, 0, INT_MAX, d_status, st)
+                                                              : tc_block_exchange(F, nodes, (int)s0, d_status, st);
                 if (rc2 != NDHSS_OK) {
                     if (d_aii) cudaFreeAsync(d_aii, st);
                     return rc2;

@@ -149,6 +149,9 @@ ndhss_status hss_ulv_level(FactorData& F, const Tree& t, int level, void* aii, c
 
 // Outer pivot block of the two-level Gauss-Jordan sweep on the tensor cores.
 constexpr int TC_KB2 = 128;
+constexpr int TC64_KB2 = 64;     // the same for FP64 fronts (tcgemm64.cu)
+constexpr int TC64_KB1 = 16;     // widest panel exchanged inside an outer block of FP64 fronts
+constexpr int TC64_INNER_MIN = 64;   // from this largest interior block of a level on
 // Whether a level whose largest interior block has mi_max unknowns takes the
 // two-level sweep with tensor-core block exchanges; tcgemm.cu.
 bool tc_front_path(const FactorData& F, int64_t mi_max);
@@ -158,6 +161,11 @@ bool tc_front_path(const FactorData& F, int64_t mi_max);
 // tcgen05 GEMM with K = the block's width; tcgemm.cu.
 ndhss_status tc_block_exchange(FactorData& F, const std::vector<int>& nodes, int k0, DevStatus* d_status,
                                cudaStream_t st);
+// The same for FP64 fronts (tcgemm64.cu): pivots [k0, min(k0 + width, m_i)) of
+// every front, exchanged on its columns [j0, min(j1, m)) -- up to m_i when j1 is
+// finite -- other than the pivots' own.
+ndhss_status tc64_block_exchange(FactorData& F, const std::vector<int>& nodes, int k0, int width, int j0, int j1,
+                                 DevStatus* d_status, cudaStream_t st);
 
 // Input and output of one apply chosen on the device (by the kernel before
 // it on the stream): the apply kernels read x and y here at their start and

@@ -65,7 +65,6 @@ constexpr int TC_PRODUCER = 256, TC_ISSUER = 288;
 constexpr int TC_HALF = TC_TILE / 2;           // columns per accumulating warp (warps w and w + 4 share lanes)
 constexpr int TC_CHUNK = 2;                    // K stages per tensor-memory accumulation chunk
 constexpr uint32_t TC_TILE_BYTES = 128u * 128u;   // 128 rows x one 128-byte swizzle row
-constexpr unsigned long long TC_WAIT_NS = 2000000000ull;
 
 // One front's part of an outer block: the slab's width w (pivots
 // [k0, k0 + w)), the first packed row row0 of its operands (A: cx m rows per
@@ -87,55 +86,11 @@ struct TcJob {
 };
 
 // ---------------------------------------------------------------- helpers
-__device__ __forceinline__ unsigned long long globaltimer() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Wait for the phase with the given parity; false when TC_WAIT_NS passed.
-__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity) {
-    const uint32_t a = tc::smem_u32(bar);
-    unsigned long long t0 = 0;
-    for (uint32_t it = 0;; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if ((it & 255u) == 0) {
-            const unsigned long long t = globaltimer();
-            if (it == 0) t0 = t;
-            else if (t - t0 > TC_WAIT_NS) return false;
-        }
-    }
-}
-
-__device__ __forceinline__ void bar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(tc::smem_u32(bar))
-        : "memory");
-}
-
-// K-major operand tile with 128-byte swizzle: 8-row groups 1024 bytes apart
-// (stride byte offset), the leading byte offset unused, layout type 2.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
+// Descriptor of a K-major operand tile with 128-byte swizzle: 8-row groups 1024
+// bytes apart (stride byte offset), the leading byte offset unused, layout
+// type 2.  Low word: start address / 16 (all of shared memory fits its field).
+constexpr uint32_t SW128_HI = (1024u >> 4) | 1u << 14 | 2u << 29;
+__device__ __forceinline__ uint32_t sw128_lo(uint32_t saddr) { return (saddr >> 4) | 1u << 16; }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
@@ -323,15 +278,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const TcJob* __restrict
     if (tid == TC_PRODUCER) {
         for (int kb = 0; kb < nk; ++kb) {
             const int s = kb % STAGES;
-            if (kb >= STAGES && !bar_wait(&empty_bar[s], ((kb / STAGES) & 1) ^ 1)) {
+            if (kb >= STAGES && !tc::bar_wait(&empty_bar[s], ((kb / STAGES) & 1) ^ 1)) {
                 atomicExch(&s_abort, 1);
                 break;
             }
             if (*(volatile int*)&s_abort) break;
-            bar_expect_tx(&full_bar[s], STAGE_BYTES);
+            tc::bar_expect_tx(&full_bar[s], STAGE_BYTES);
             for (int p = 0; p < NS; ++p) {
-                tma_load_2d(tileA(s, p), &tmap, kb * BK, J.a_row + p * J.a_pstride + m0, &full_bar[s]);
-                tma_load_2d(tileB(s, p), &tmap, kb * BK, J.b_row + p * J.b_pstride + n0, &full_bar[s]);
+                tc::tma_load_2d(tileA(s, p), &tmap, kb * BK, J.a_row + p * J.a_pstride + m0, &full_bar[s]);
+                tc::tma_load_2d(tileB(s, p), &tmap, kb * BK, J.b_row + p * J.b_pstride + n0, &full_bar[s]);
             }
             issued = kb + 1;
         }
@@ -340,7 +295,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const TcJob* __restrict
         bool ok = true;
         for (int c = 0; c < nchunk && ok; ++c) {
             const int b = c & 1;
-            if (c >= 2 && !bar_wait(&accfree_bar[b], ((c >> 1) & 1) ^ 1)) {
+            if (c >= 2 && !tc::bar_wait(&accfree_bar[b], ((c >> 1) & 1) ^ 1)) {
                 ok = false;
                 break;
             }
@@ -349,21 +304,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const TcJob* __restrict
             const int kb1 = min(nk, (c + 1) * TC_CHUNK);
             for (int kb = c * TC_CHUNK; kb < kb1; ++kb) {
                 const int s = kb % STAGES;
-                if (!bar_wait(&full_bar[s], (kb / STAGES) & 1)) {
+                if (!tc::bar_wait(&full_bar[s], (kb / STAGES) & 1)) {
                     ok = false;
                     break;
                 }
                 tc::fence_after();
+                const uint32_t lo = sw128_lo(tileA(s, 0));
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
 #pragma unroll
                     for (int q = 0; q < NP; ++q) {
-                        const uint64_t ad = sw128_desc(tileA(s, prod_a(q)) + 32u * kk);
-                        const uint64_t bd = sw128_desc(tileB(s, prod_b(q)) + 32u * kk);
+                        const uint32_t ad = lo + (uint32_t)prod_a(q) * (TC_TILE_BYTES >> 4) + 2u * kk;
+                        const uint32_t bd = lo + (uint32_t)(NS + prod_b(q)) * (TC_TILE_BYTES >> 4) + 2u * kk;
                         const uint32_t d = q == 0 ? acc0 : acc0 + (uint32_t)TC_TILE;
                         const uint32_t acc = (kb != c * TC_CHUNK || kk != 0 || q >= 2) ? 1u : 0u;
-                        if constexpr (ESZ == 4) tc::mma_tf32(d, ad, bd, idesc, acc);
-                        else tc::mma_f16(d, ad, bd, idesc, acc);
+                        if constexpr (ESZ == 4) tc::mma_tf32(d, ad, bd, SW128_HI, idesc, acc);
+                        else tc::mma_f16(d, ad, bd, SW128_HI, idesc, acc);
                     }
                 }
                 tc::commit(&empty_bar[s]);
@@ -372,7 +328,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const TcJob* __restrict
         }
         if (!ok) atomicExch(&s_abort, 1);
         tc::commit(&done_bar);                        // fires once every MMA issued above has retired
-        bar_wait(&done_bar, 0);
+        tc::bar_wait(&done_bar, 0);
     } else if (warp < 8) {
         // accumulating warps: each finished chunk pair of this thread's TMEM
         // lane (real row m0 + rr of the product) is added into FP32 registers
@@ -387,7 +343,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const TcJob* __restrict
         bool ok = true;
         for (int c = 0; c < nchunk; ++c) {
             const int b = c & 1;
-            if (!bar_wait(&accfull_bar[b], (c >> 1) & 1)) {
+            if (!tc::bar_wait(&accfull_bar[b], (c >> 1) & 1)) {
                 ok = false;
                 break;
             }
@@ -469,7 +425,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap, const TcJob* __restrict
     // leave only once every copy issued by this CTA has landed
     if (tid == TC_PRODUCER) {
         for (int kb = max(0, issued - STAGES); kb < issued; ++kb)
-            if (!bar_wait(&full_bar[kb % STAGES], (kb / STAGES) & 1)) break;
+            if (!tc::bar_wait(&full_bar[kb % STAGES], (kb / STAGES) & 1)) break;
     }
     tc::fence_before();
     __syncthreads();
@@ -521,13 +477,13 @@ ndhss_status tc_block_run(FactorData& F, const std::vector<int>& nodes, int k0, 
     TcJob* d_jobs = reinterpret_cast<TcJob*>(buf + packed_bytes + fr_bytes);
     int2* d_t = reinterpret_cast<int2*>(buf + packed_bytes + fr_bytes + job_bytes);
     ndhss_status rc = NDHSS_OK;
-    auto cp = [&](void* dst, const void* src, size_t b) {
-        if (rc == NDHSS_OK && cudaMemcpyAsync(dst, src, b, cudaMemcpyHostToDevice, st) != cudaSuccess)
-            rc = set_error(NDHSS_ERR_CUDA, "ndhss_factor: upload of the tensor-core tables failed");
-    };
-    cp(d_fr, fr.data(), fr.size() * sizeof(TcFront));
-    cp(d_jobs, jobs.data(), jobs.size() * sizeof(TcJob));
-    cp(d_t, tiles.data(), tiles.size() * sizeof(int2));
+    // the three tables in one copy
+    std::vector<unsigned char> tab(fr_bytes + job_bytes + t_bytes);
+    std::memcpy(tab.data(), fr.data(), fr.size() * sizeof(TcFront));
+    std::memcpy(tab.data() + fr_bytes, jobs.data(), jobs.size() * sizeof(TcJob));
+    std::memcpy(tab.data() + fr_bytes + job_bytes, tiles.data(), tiles.size() * sizeof(int2));
+    if (cudaMemcpyAsync(d_fr, tab.data(), tab.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        rc = set_error(NDHSS_ERR_CUDA, "ndhss_factor: upload of the tensor-core tables failed");
     CUtensorMap tmap;
     if (rc == NDHSS_OK) {
         const cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)rows};
@@ -591,11 +547,10 @@ bool tc_front_path(const FactorData& F, int64_t mi_max) {
     // the two-level sweep (default 96; smaller fronts leave the blocks and
     // 128 x 128 tiles mostly empty); NDHSS_FRONT_UPDATE=simt keeps every
     // level on the rank-kb sweep over whole fronts (CUDA cores; a cross-check)
-    if (F.prec == NDHSS_FP64) return false;
     const char* u = std::getenv("NDHSS_FRONT_UPDATE");
     if (u && std::strcmp(u, "simt") == 0) return false;
     const char* e = std::getenv("NDHSS_TC_MIN_MI");
-    const int min_mi = e ? std::atoi(e) : 96;
+    const int min_mi = e ? std::atoi(e) : F.prec == NDHSS_FP64 ? 24 : 96;
     return min_mi > 0 && mi_max >= min_mi;
 }
 

@@ -58,19 +58,24 @@ __device__ __forceinline__ uint32_t core_off16(int r, int k, int K) {
            (uint32_t)(k & 7) * 2u;
 }
 
-// one kind::f16 MMA (K = 16 for 16-bit operands: the start addresses advance 256 bytes per step)
-__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+// One MMA of kind::f16 (K = 16 for 16-bit operands) or kind::tf32 (K = 8).  The
+// operands' shared-memory descriptors come as words: the low word (start
+// address and leading byte offset) is a base plus a constant per operand tile
+// and K step, the high word the same for all, so the issuing thread spends an
+// addition per operand (building 64-bit descriptors for every MMA took it about
+// 100 clocks, more than the MMA itself).
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+        "{\n.reg .pred p;\n.reg .b64 a, b;\nsetp.ne.b32 p, %5, 0;\nmov.b64 a, {%1, %3};\nmov.b64 b, {%2, %3};\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n}\n" ::"r"(tmem_d),
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(acc));
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+        "{\n.reg .pred p;\n.reg .b64 a, b;\nsetp.ne.b32 p, %5, 0;\nmov.b64 a, {%1, %3};\nmov.b64 b, {%2, %3};\n"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %4, p;\n}\n" ::"r"(tmem_d),
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(acc));
 }
 
 __device__ __forceinline__ void commit(uint64_t* mbar) {
@@ -108,6 +113,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, int m
     return done != 0;
 }
 
+// the same without the wait: the values are valid after tmem_wait_ld
+__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// (after tmem_wait_ld) keeps the compiler from using the values before the wait
+__device__ __forceinline__ void tmem_landed(uint32_t (&r)[8]) {
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+}
+
 // eight consecutive 32-bit columns of this thread's TMEM lane (warp w reads
 // lanes 32 w .. 32 w + 31: taddr carries the lane offset in bits 16..31)
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
@@ -118,6 +135,47 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(r[u]);
+}
+
+// Bounded waits: how long, and the clock
+constexpr unsigned long long WAIT_NS = 2000000000ull;
+__device__ __forceinline__ unsigned long long globaltimer() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// Wait for the phase with the given parity; false when WAIT_NS passed.
+__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity) {
+    const uint32_t a = smem_u32(bar);
+    unsigned long long t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(a), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if ((it & 255u) == 0) {
+            const unsigned long long t = globaltimer();
+            if (it == 0) t0 = t;
+            else if (t - t0 > WAIT_NS) return false;
+        }
+    }
+}
+
+__device__ __forceinline__ void bar_expect_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* map, int x, int y, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+            dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
+        : "memory");
 }
 
 }  // namespace tc
