@@ -62,38 +62,53 @@ template <> __device__ __forceinline__ c64 shfl_idx<c64>(c64 v, int src) {
 // F = blockdiag(S^mu, S^nu) scattered to the parent order of Eq. 3.4 (zero
 // where the row and column come from different children).  fsrc[pos] =
 // (child << 30) | row of that child's S.
+//
+// Bound by memory: a warp takes a column at a time with four rows per lane in
+// flight, ASM_COLS columns per CTA.  (A CTA per column left most of its 256
+// threads without a row in the small fronts, a million CTAs on the leaf level
+// of a 512 x 512 P2 problem: 6.9 ms per factorization, 1.9 ms so.)
+constexpr int ASM_COLS = 32;
 template <typename T>
-__global__ void assemble_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ node,
-                                const int64_t* __restrict__ foff, const int32_t* __restrict__ fsrc,
-                                const int64_t* __restrict__ poff, T* __restrict__ front) {
+__global__ void __launch_bounds__(256)
+assemble_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ node, const int64_t* __restrict__ foff,
+                const int32_t* __restrict__ fsrc, const int64_t* __restrict__ poff, T* __restrict__ front) {
     const int s = lev[blockIdx.y];
-    const int64_t m = nf(node, s, 5) + nf(node, s, 7);
+    const int m = nf(node, s, 5) + nf(node, s, 7);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     T* F = front + foff[s];
     const int c0 = nf(node, s, 2);
-    if (c0 < 0) {
-        for (int64_t c = blockIdx.x; c < m; c += gridDim.x)
-            for (int64_t r = threadIdx.x; r < m; r += blockDim.x) F[c * m + r] = zero<T>();
-        return;
-    }
-    const int ch[2] = {c0, nf(node, s, 3)};
-    const T* CF[2];
-    int64_t cm[2], cmi[2];
-    for (int w = 0; w < 2; ++w) {
-        cmi[w] = nf(node, ch[w], 5);
-        cm[w] = cmi[w] + nf(node, ch[w], 7);
-        CF[w] = front + foff[ch[w]];
-    }
+    const bool leaf = c0 < 0;
+    const T* CS[2] = {nullptr, nullptr};       // S of the children, column-major with ld cm
+    int64_t cm[2] = {0, 0};
+    if (!leaf)
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const int ch = w ? nf(node, s, 3) : c0;
+            const int64_t cmi = nf(node, ch, 5);
+            cm[w] = cmi + nf(node, ch, 7);
+            CS[w] = front + foff[ch] + cmi * cm[w] + cmi;
+        }
     const int32_t* src = fsrc + poff[s];
-    for (int64_t c = blockIdx.x; c < m; c += gridDim.x) {
-        const int sc = src[c];
+    const int cend = min(m, ((int)blockIdx.x + 1) * ASM_COLS);
+    for (int c = blockIdx.x * ASM_COLS + warp; c < cend; c += 8) {
+        T* Fc = F + (int64_t)c * m;
+        const int sc = leaf ? 0 : src[c];
         const int wc = sc >> 30;
-        const int64_t lc = sc & 0x3fffffff;
-        const T* colS = CF[wc] + (cmi[wc] + lc) * cm[wc] + cmi[wc];
-        for (int64_t r = threadIdx.x; r < m; r += blockDim.x) {
-            const int sr = src[r];
-            T v = zero<T>();
-            if ((sr >> 30) == wc) v = colS[sr & 0x3fffffff];
-            F[c * m + r] = v;
+        const T* colS = leaf ? nullptr : (wc ? CS[1] : CS[0]) + (int64_t)(sc & 0x3fffffff) * (wc ? cm[1] : cm[0]);
+        for (int r0 = lane; r0 < m; r0 += 128) {
+            int sr[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = r0 + 32 * u;
+                sr[u] = (!leaf && r < m) ? src[r] : -1;
+            }
+            T v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                v[u] = (sr[u] >= 0 && (sr[u] >> 30) == wc) ? colS[sr[u] & 0x3fffffff] : zero<T>();
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (r0 + 32 * u < m) Fc[r0 + 32 * u] = v[u];
         }
     }
 }
@@ -1051,7 +1066,7 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
             mimax = std::max<int64_t>(mimax, F.m_i(s));
         }
         if (mmax == 0) continue;
-        const int agx = (int)std::min<int64_t>(mmax, 256);
+        const unsigned agx = (unsigned)((mmax + ASM_COLS - 1) / ASM_COLS);
         tm.begin();
         for (int c0 = 0; c0 < L; c0 += MAX_GRID_YZ) {
             assemble_kernel<T><<<dim3(agx, std::min(MAX_GRID_YZ, L - c0)), 256, 0, st>>>(lev + c0, F.d_node, F.d_foff,
