@@ -24,6 +24,7 @@
 #include <cmath>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -81,6 +82,13 @@ __device__ __forceinline__ float shfl_xor_h(float v, int o) { return __shfl_xor_
 template <typename R>
 __device__ __forceinline__ Cx<R> shfl_xor_h(Cx<R> v, int o) {
     return {__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
+}
+
+__device__ __forceinline__ double shfl_from(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ float shfl_from(float v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+template <typename R>
+__device__ __forceinline__ Cx<R> shfl_from(Cx<R> v, int l) {
+    return {__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l)};
 }
 
 __host__ __device__ __forceinline__ int rows_cap_even(int r) { return (r + 1) & ~1; }
@@ -635,21 +643,52 @@ row_id_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, T* 
 // thread-block cluster (C = 1: one CTA), every CTA holding its share in shared
 // memory.  A pivot step is one cluster barrier (the CTAs' per-warp candidates
 // of the next pivot become visible and every warp reduces them through
-// distributed shared memory), the copy of the pivot column from its owner, one
-// CTA barrier and the reflection of the remaining local columns, which also
-// yields their new norms and the next candidates.  A column is reflected by a
-// segment of LPC lanes (LPC = 8, 16 or 32 as p <= 64, 128, 256; 8 entries per
-// lane), so a warp works on 32 / LPC columns at once.  Columns never move: a
-// pivot is flagged, the pivot order kept, and R11 = R(0:k, 0:k) gathered at
-// the end.  Ties of the pivot norm go to the lowest row index.
-constexpr int RID_THREADS = 256;
-constexpr int RID_NW = RID_THREADS / 32;
+// distributed shared memory) and the reflection of the remaining local
+// columns, which also yields their new norms and the next candidates; the
+// pivot column is read in place.  A column is handled by a segment of LPC lanes
+// with CH entries each (rid_shape), so a warp works on 32 / LPC columns at
+// once.  Columns never move: a pivot is flagged and the pivot order kept.
+// Ties of the pivot norm go to the lowest row index.
+//
+// The rows above the pivot carry T = R11^{-1} R12 along: when row t of R is
+// final, r = R(t, c) / R(t, t) gives T(t, c) = r and T(0:t, c) -= T(0:t, piv) r,
+// in entries that the step holds in registers anyway, so no triangular solve
+// follows (one thread per column, k^2 / 2 dependent shared-memory reads: about
+// half of the kernel at ranks near 100).  Entries lie at row sl + LPC q, so
+// only the slots q >= t / LPC take part in the dot product and the norm; the
+// step is instantiated per first slot, since a predicated-off FMA costs as
+// much as one that runs.
+//
+// Before and after this form (64 registers, 8 entries per lane always, 128
+// columns per CTA before): factorization of a 192 x 192 elastic matrix (ranks to
+// 112) 64 -> 35 ms, row IDs of a 256 x 256 P2 Helmholtz factor 13.1 -> 10.5 ms in
+// complex64 and 78 -> 44 ms in complex128.  What bounds it now: per pivot the
+// barrier, two remote reads and the scalars (~1.2 us) in FP32, the FP64 pipe in
+// FP64.
+template <typename T> struct Rid {
+    static constexpr bool fp64 = sizeof(typename Tr<T>::real) == 8;
+    // FP64: one warp per SM quarter already fills its FP64 pipe
+    static constexpr int THREADS = fp64 ? 128 : 256;
+    static constexpr int NW = THREADS / 32;
+    // a node is split down to this many columns per CTA while the launch still
+    // fits SPLIT_CTAS CTAs per SM
+    static constexpr int SPLIT_COLS = 32;
+    static constexpr int SPLIT_CTAS = fp64 ? 4 : 2;
+};
 constexpr int RID_KMAX = 256;                 // ranks stay below the 256-sample limit
-constexpr int RID_MAX_CLUSTER = 8;
+constexpr int RID_MAX_CLUSTER = 16;           // largest cluster (beyond the portable 8 only to fit shared memory)
+constexpr int RID_SPLIT_CLUSTER = 8;          // largest cluster taken for speed
 constexpr size_t RID_SMEM = 200 * 1024;       // dynamic shared memory of one CTA's share
-constexpr int RID_SPLIT_COLS = 128;
 
-__host__ __device__ __forceinline__ int rid_lpc(int p) { return p <= 64 ? 8 : p <= 128 ? 16 : 32; }
+// lanes per column and entries per lane for p samples: LPC CH >= p
+struct RidShape {
+    int lpc, ch;
+};
+__host__ __device__ __forceinline__ RidShape rid_shape(int p) {
+    const int lpc = p <= 64 ? 8 : p <= 128 ? 16 : 32;
+    const int ch = (p + lpc - 1) / lpc;
+    return {lpc, ch <= 5 ? 5 : ch};
+}
 
 template <typename T>
 __device__ __forceinline__ T seg_sum(T v, int lpc) {
@@ -657,14 +696,14 @@ __device__ __forceinline__ T seg_sum(T v, int lpc) {
     return v;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(RID_THREADS, sizeof(T) > 8 ? 2 : 4)
+template <typename T, int CH>
+__global__ void __launch_bounds__(Rid<T>::THREADS, sizeof(T) > 8 ? 3 : 2)
 row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, T* __restrict__ ws,
                       int* __restrict__ iws, int* __restrict__ kk, const int* __restrict__ rows_in, double eps,
                       int rank_cap) {
     using real = typename Tr<T>::real;
     namespace cg = cooperative_groups;
-    constexpr int CH = 8;                        // column entries per lane in registers
+    constexpr int NT = Rid<T>::THREADS, NW = Rid<T>::NW;
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks();
     const int rk = (int)cl.block_rank();
@@ -676,21 +715,20 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
     const int nloc = min(rows, c_lo + chunk) - c_lo;
     const int lds = p | 1;                       // odd column stride: per-column loops free of bank conflicts
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int lpc = rid_lpc(p), spw = 32 / lpc;  // lanes per column, columns per warp
+    const int lpc = rid_shape(p).lpc, spw = 32 / lpc;  // lanes per column, columns per warp
     const int seg = lane / lpc, sl = lane % lpc;
     extern __shared__ __align__(16) unsigned char smem[];
     T* Ws = reinterpret_cast<T*>(smem);          // nloc columns of W, ld lds
     unsigned char* used = reinterpret_cast<unsigned char*>(Ws + (size_t)lds * chunk + p + 1);
-    __shared__ real s_cv[2][RID_NW];
-    __shared__ int s_ci[2][RID_NW];
-    __shared__ T s_beta[RID_KMAX];
+    __shared__ real s_cv[2][NW];
+    __shared__ int s_ci[2][NW];
     __shared__ int s_order[RID_KMAX];
     const T* Wg = ws + nd.o_w;
-    for (int q = tid; q < p * nloc; q += RID_THREADS) {
+    for (int q = tid; q < p * nloc; q += NT) {
         const int c = q / p, j = q % p;
         Ws[(size_t)c * lds + j] = Wg[(int64_t)(c_lo + c) * p + j];
     }
-    for (int c = tid; c < nloc; c += RID_THREADS) used[c] = 0;
+    for (int c = tid; c < nloc; c += NT) used[c] = 0;
     __syncthreads();
     // the warp's best candidate (squared norm, row) over its segments, to s_cv/s_ci[par]
     auto publish = [&](real best, int nb, int par) {
@@ -701,7 +739,7 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
     {
         real best = real(-1);
         int nb = INT_MAX;
-        for (int c0 = warp * spw; c0 < nloc; c0 += RID_NW * spw) {
+        for (int c0 = warp * spw; c0 < nloc; c0 += NW * spw) {
             const int c = c0 + seg;
             const bool act = c < nloc;
             const T* col = Ws + (size_t)(act ? c : 0) * lds;
@@ -713,7 +751,7 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
         publish(best, nb, 0);
     }
     const int kmax = min(min(min(nd.kcap, rank_cap), min(p, rows)), RID_KMAX);
-    // pivot scalars in the working precision, computed by every thread (no
+    // pivot scalars in the working precision, computed by every warp (no
     // broadcast barrier; double would run on the narrow FP64 pipe)
     real r11 = real(0);
     const real reps = (real)eps;
@@ -723,8 +761,8 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
         const int par = t & 1;
         real bv = real(-1);
         int bi = INT_MAX;
-        for (int q = lane; q < C * RID_NW; q += 32) {
-            const int r = q / RID_NW, w = q % RID_NW;
+        for (int q = lane; q < C * NW; q += 32) {
+            const int r = q / NW, w = q % NW;
             real v;
             int i;
             if (C > 1) {
@@ -741,9 +779,17 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
             bi = warp_argmax(bv, bi, bi != INT_MAX, &gv);
             bv = gv;
         }
-        const real xn = sqrt(bv > real(0) ? bv : real(0));
-        if (t == 0) r11 = xn;
-        if (t >= kmax || bi == INT_MAX || !(xn > reps * r11)) break;
+        // ||x|| > eps R(0, 0), compared as squares in FP64 (a square root there is
+        // a long sequence on the FP64 pipe)
+        real xn = real(0);
+        if constexpr (Rid<T>::fp64) {
+            if (t == 0) r11 = bv;
+            if (t >= kmax || bi == INT_MAX || !(bv > reps * reps * r11)) break;
+        } else {
+            xn = sqrt(bv > real(0) ? bv : real(0));
+            if (t == 0) r11 = xn;
+            if (t >= kmax || bi == INT_MAX || !(xn > reps * r11)) break;
+        }
         const int cb = bi, owner = cb / chunk;
         // the pivot column, read in place by every thread (local or through
         // distributed shared memory): no step writes it from here on
@@ -753,80 +799,87 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
             s_order[t] = cb;
             if (owner == rk) used[cb - c_lo] = 1;    // read from the next step on (after its barrier)
         }
-        // reflector v = x - beta e_t of the pivot column x, beta = -phase(x_t) ||x||
+        // reflector v = x - beta e_t of the pivot column's rows x from t on,
+        // beta = -phase(x_t) ||x||; 2 / |v|^2 = 1 / (||x|| (||x|| + |x_t|))
         const T a0 = src[t];
-        const real aa2 = nrm2r(a0), aa = sqrt(aa2);
-        T ph = one<T>();
-        if (aa > real(0)) ph = scale(a0, real(1) / aa);
-        const T beta = scale(ph, -xn);
-        const T v0 = a0 - beta;
-        const real vn2 = xn * xn - aa2 + nrm2r(v0);
-        if (tid == 0) s_beta[t] = beta;
-        const real f = real(2) / vn2;
-        T vl[CH];
+        const real aa2 = nrm2r(a0);
+        real aa, rxn, raa;
+        if constexpr (Rid<T>::fp64) {
+            // both inverse roots in one sequence: even lanes ||x||, odd lanes |x_t|
+            const real rs = rsqrt((lane & 1) ? aa2 : bv);
+            rxn = shfl_from(rs, 0);
+            raa = shfl_from(rs, 1);
+            xn = bv * rxn;
+            aa = aa2 > real(0) ? aa2 * raa : real(0);
+        } else {
+            aa = sqrt(aa2);
+            rxn = real(1) / xn;
+            raa = real(1) / aa;
+        }
+        const T ph = aa > real(0) ? scale(a0, raa) : one<T>();
+        const T v0 = a0 + scale(ph, xn);
+        const real f = rxn / (xn + aa);
+        const T rbeta = -scale(conjv(ph), rxn);      // 1 / R(t, t)
+        // z: rows below t, the reflector; rows above, T of the pivot column
+        T z[CH];
 #pragma unroll
         for (int q = 0; q < CH; ++q) {
-            const int j = t + sl + lpc * q;
-            vl[q] = (j < p) ? (j == t ? v0 : src[j]) : zero<T>();
+            const int j = sl + lpc * q;
+            z[q] = (j < p) ? (j == t ? v0 : src[j]) : zero<T>();
         }
         real best = real(-1);
         int nb = INT_MAX;
-        for (int c0 = warp * spw; c0 < nloc; c0 += RID_NW * spw) {
-            const int c = c0 + seg;
-            const bool act = c < nloc && !used[c] && c_lo + c != cb;
-            T* col = Ws + (size_t)(act ? c : 0) * lds;
-            T cv[CH];
-            T w = zero<T>();
+        auto reflect = [&](auto qtc) {
+            constexpr int QT = decltype(qtc)::value;  // the slot of row t
+            const bool lowt = sl + lpc * QT < t, is_t = sl + lpc * QT == t;
+            for (int c0 = warp * spw; c0 < nloc; c0 += NW * spw) {
+                const int c = c0 + seg;
+                const bool act = c < nloc && !used[c] && c_lo + c != cb;
+                T* col = Ws + (size_t)(act ? c : 0) * lds;
+                T cv[CH];
 #pragma unroll
-            for (int q = 0; q < CH; ++q) {
-                const int j = t + sl + lpc * q;
-                cv[q] = (act && j < p) ? col[j] : zero<T>();
-            }
-#pragma unroll
-            for (int q = 0; q < CH; ++q) w = fmac(conjv(vl[q]), cv[q], w);
-            w = seg_sum(w, lpc);
-            const T g = scale(w, f);
-            real sacc = real(0);
-#pragma unroll
-            for (int q = 0; q < CH; ++q) {
-                const int j = t + sl + lpc * q;
-                if (act && j < p) {
-                    const T u = cv[q] - vl[q] * g;
-                    col[j] = u;
-                    if (j > t) sacc += nrm2r(u);
+                for (int q = 0; q < CH; ++q) {
+                    const int j = sl + lpc * q;
+                    cv[q] = (act && j < p) ? col[j] : zero<T>();
                 }
+                const T ct = shfl_from(cv[QT], seg * lpc + t - lpc * QT);
+                T w = fmac(conjv(lowt ? zero<T>() : z[QT]), cv[QT], zero<T>());
+#pragma unroll
+                for (int q = QT + 1; q < CH; ++q) w = fmac(conjv(z[q]), cv[q], w);
+                w = seg_sum(w, lpc);
+                const T g = scale(w, f);
+                const T h = (ct - v0 * g) * rbeta;    // row t of T
+                real sacc = real(0);
+#pragma unroll
+                for (int q = 0; q < CH; ++q) {
+                    const int j = sl + lpc * q;
+                    T u = cv[q] - z[q] * ((q < QT || (q == QT && lowt)) ? h : g);
+                    if (q == QT && is_t) u = h;
+                    if (act && j < p) col[j] = u;
+                    if (q > QT || (q == QT && !lowt && !is_t)) sacc += nrm2r(u);
+                }
+                sacc = seg_sum(sacc, lpc);
+                if (act && sacc > best) { best = sacc; nb = c_lo + c; }
             }
-            sacc = seg_sum(sacc, lpc);
-            if (act && sacc > best) { best = sacc; nb = c_lo + c; }
+        };
+        switch (t / lpc) {
+            case 0: reflect(std::integral_constant<int, 0>{}); break;
+            case 1: reflect(std::integral_constant<int, 1>{}); break;
+            case 2: reflect(std::integral_constant<int, 2>{}); break;
+            case 3: reflect(std::integral_constant<int, 3>{}); break;
+            case 4: reflect(std::integral_constant<int, 4>{}); break;
+            case 5: reflect(std::integral_constant<int, (CH > 5 ? 5 : 0)>{}); break;
+            case 6: reflect(std::integral_constant<int, (CH > 6 ? 6 : 0)>{}); break;
+            default: reflect(std::integral_constant<int, (CH > 7 ? 7 : 0)>{}); break;
         }
         publish(best, nb, par ^ 1);
     }
     const int k = t;
-    // R11 stays in the pivot columns, in the shared memory of their owners
-    // (the pivot columns are not written below): one pointer per column,
-    // local or through distributed shared memory
-    __shared__ const T* s_pcol[RID_KMAX];
-    for (int a = tid; a < k; a += RID_THREADS) {
-        const int cb = s_order[a], owner = cb / chunk;
-        s_pcol[a] = (owner == rk) ? Ws + (size_t)(cb - c_lo) * lds
-                                  : cl.map_shared_rank(Ws, owner) + (size_t)(cb - owner * chunk) * lds;
-    }
-    if (C > 1) cl.sync(); else __syncthreads();
-    // T = R11^{-1} R12 in place of R12 (one column per thread)
-    for (int c = tid; c < nloc; c += RID_THREADS) {
-        if (used[c]) continue;
-        T* col = Ws + (size_t)c * lds;
-        for (int i = k - 1; i >= 0; --i) {
-            T acc = col[i];
-            for (int l = i + 1; l < k; ++l) acc = fmac(-s_pcol[l][i], col[l], acc);
-            col[i] = acc * recip(s_beta[i]);
-        }
-    }
     // no CTA leaves while another may still read its pivot columns
     if (C > 1) cl.sync(); else __syncthreads();
     T* X = ws + nd.o_x;
     int* piv = iws + nd.o_piv;
-    for (int q = tid; q < nloc * k; q += RID_THREADS) {
+    for (int q = tid; q < nloc * k; q += NT) {
         const int c = q % nloc, a = q / nloc;
         T v;
         if (used[c]) v = (s_order[a] == c_lo + c) ? one<T>() : zero<T>();
@@ -835,8 +888,8 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
     }
     // piv: skeleton in pivot order, then the other rows in increasing order
     if (rk == 0)
-        for (int a = tid; a < k; a += RID_THREADS) piv[a] = s_order[a];
-    for (int c = tid; c < nloc; c += RID_THREADS) {
+        for (int a = tid; a < k; a += NT) piv[a] = s_order[a];
+    for (int c = tid; c < nloc; c += NT) {
         if (used[c]) continue;
         int below = 0;
         for (int a = 0; a < k; ++a) below += (s_order[a] < c_lo + c) ? 1 : 0;
@@ -845,7 +898,6 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
     if (rk == 0 && tid == 0) kk[id] = k;
 }
 
-// Omega_i = X^T Omega_loc, S_i = S_loc(J, :), skeleton = iloc(J).
 template <typename T>
 __global__ void __launch_bounds__(HT)
 finish_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, const HFront* __restrict__ fronts,
@@ -1674,7 +1726,18 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
         const int w_in_smem = smem_w <= 200 * 1024 ? 1 : 0;
         (void)w_in_smem;
         HSS_TRY(cudaFuncSetAttribute(row_id_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem_base, 48 * 1024)));
-        HSS_TRY(cudaFuncSetAttribute(row_id_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RID_SMEM));
+        // the cluster kernel's instance for this round's sample count
+        using RidKernel = void (*)(const int*, const HNode*, T*, int*, int*, const int*, double, int);
+        const RidKernel rid_kernel = [](int ch) -> RidKernel {
+            switch (ch) {
+                case 5: return row_id_cluster_kernel<T, 5>;
+                case 6: return row_id_cluster_kernel<T, 6>;
+                case 7: return row_id_cluster_kernel<T, 7>;
+                default: return row_id_cluster_kernel<T, 8>;
+            }
+        }(rid_shape(p).ch);
+        HSS_TRY(cudaFuncSetAttribute(rid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RID_SMEM));
+        HSS_TRY(cudaFuncSetAttribute(rid_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         // row IDs of the nodes flat[b, e): the cluster kernel with the smallest
         // cluster whose share of W fits in shared memory, one launch per cluster
         // size; a node too large for RID_MAX_CLUSTER CTAs keeps W in global memory
@@ -1687,29 +1750,33 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
         HSS_TRY(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
         auto launch_row_id = [&](size_t b, size_t e) -> ndhss_status {
             std::vector<int> grp[5], big;
-            // a node whose share would exceed RID_SPLIT_COLS columns per CTA is
-            // split further (its pivot steps run shorter) when all such nodes
-            // together take at most two CTAs per SM: the launch lasts as long
-            // as its longest pivot chain
+            // a node is split down to SPLIT_COLS columns per CTA (its pivot steps
+            // run shorter: the launch lasts as long as its longest pivot chain),
+            // or to the smallest power-of-two multiple of that for which all
+            // nodes together still take at most SPLIT_CTAS CTAs per SM
             auto g_fit = [&](int rc) {
                 int g = 0;
                 while ((1 << g) <= RID_MAX_CLUSTER && rid_bytes(rc, 1 << g) > RID_SMEM) ++g;
                 return g;
             };
-            auto g_split = [&](int rc, int g) {
-                while ((1 << g) < RID_MAX_CLUSTER && (rc + (1 << g) - 1) / (1 << g) > RID_SPLIT_COLS) ++g;
+            auto g_split = [&](int rc, int cols) {
+                int g = g_fit(rc);
+                while ((1 << g) < RID_SPLIT_CLUSTER && (rc + (1 << g) - 1) / (1 << g) > cols) ++g;
                 return g;
             };
-            int64_t split_ctas = 0;
-            for (size_t q = b; q < e; ++q) {
-                const int rc = nodes[flat[q]].rows_cap, g0 = g_fit(rc);
-                if (g0 > 0 || g_split(rc, g0) > g0) split_ctas += (int64_t)1 << g_split(rc, g0);
+            int cols = Rid<T>::SPLIT_COLS;
+            for (;; cols *= 2) {
+                int64_t ctas = 0;
+                int rcmax = 0;
+                for (size_t q = b; q < e; ++q) {
+                    const int rc = nodes[flat[q]].rows_cap;
+                    rcmax = std::max(rcmax, rc);
+                    ctas += (int64_t)1 << g_split(rc, cols);
+                }
+                if (ctas <= (int64_t)Rid<T>::SPLIT_CTAS * num_sms || cols >= rcmax) break;
             }
-            const bool split = split_ctas <= 2 * (int64_t)num_sms;
             for (size_t q = b; q < e; ++q) {
-                const int rc = nodes[flat[q]].rows_cap;
-                int g = g_fit(rc);
-                if (split && (1 << g) <= RID_MAX_CLUSTER) g = g_split(rc, g);
+                const int g = g_split(nodes[flat[q]].rows_cap, cols);
                 ((1 << g) <= RID_MAX_CLUSTER ? grp[g] : big).push_back(flat[q]);
             }
             // a cluster shape the device cannot co-schedule falls back to global memory
@@ -1717,7 +1784,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                 if (grp[g].empty()) continue;
                 cudaLaunchConfig_t cfg{};
                 cfg.gridDim = dim3((unsigned)(1 << g));
-                cfg.blockDim = dim3(RID_THREADS);
+                cfg.blockDim = dim3(Rid<T>::THREADS);
                 cfg.dynamicSmemBytes = RID_SMEM;
                 cudaLaunchAttribute at[1];
                 at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1727,7 +1794,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                 cfg.attrs = at;
                 cfg.numAttrs = 1;
                 int ncl = 0;
-                if (cudaOccupancyMaxActiveClusters(&ncl, row_id_cluster_kernel<T>, &cfg) != cudaSuccess || ncl < 1) {
+                if (cudaOccupancyMaxActiveClusters(&ncl, rid_kernel, &cfg) != cudaSuccess || ncl < 1) {
                     cudaGetLastError();
                     big.insert(big.end(), grp[g].begin(), grp[g].end());
                     grp[g].clear();
@@ -1753,12 +1820,12 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                 HSS_TRY(fork.start(li - 1));
                 const size_t sm = rid_bytes(rcmax, C);
                 if (C == 1) {
-                    row_id_cluster_kernel<T><<<(unsigned)grp[g].size(), RID_THREADS, sm, ls>>>(dl.p, dnodes.p, ws.p, iws.p,
-                                                                                              kk.p, rows.p, eps, rank_cap);
+                    rid_kernel<<<(unsigned)grp[g].size(), Rid<T>::THREADS, sm, ls>>>(dl.p, dnodes.p, ws.p, iws.p, kk.p,
+                                                                                     rows.p, eps, rank_cap);
                 } else {
                     cudaLaunchConfig_t cfg{};
                     cfg.gridDim = dim3((unsigned)(grp[g].size() * C));
-                    cfg.blockDim = dim3(RID_THREADS);
+                    cfg.blockDim = dim3(Rid<T>::THREADS);
                     cfg.dynamicSmemBytes = sm;
                     cfg.stream = ls;
                     cudaLaunchAttribute at[1];
@@ -1768,7 +1835,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                     at[0].val.clusterDim.z = 1;
                     cfg.attrs = at;
                     cfg.numAttrs = 1;
-                    HSS_TRY(cudaLaunchKernelEx(&cfg, row_id_cluster_kernel<T>, (const int*)dl.p, (const HNode*)dnodes.p,
+                    HSS_TRY(cudaLaunchKernelEx(&cfg, rid_kernel, (const int*)dl.p, (const HNode*)dnodes.p,
                                                ws.p, iws.p, kk.p, (const int*)rows.p, eps, rank_cap));
                 }
                 NDHSS_LAUNCH_CHECK("row_id_cluster_kernel");
