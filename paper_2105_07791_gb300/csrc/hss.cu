@@ -185,15 +185,27 @@ struct GemmJob {
     int realB = 0;                // complex T: B holds real values (zero imaginary parts); 2 FMAs per product
 };
 
-// 64 x 64 tiles of every job; blockIdx.z = job * ksplit + split.  The K
+// Output tiles (TILE x TILE, 256 threads with PT x PT products each).  FP64
+// products are bound by the FP64 pipe (two DFMA per clock and SM: one complex
+// 64 x 64 tile with K = 64 occupies an SM for 250 us), so FP64 takes small
+// tiles: more SMs with work, and fewer products spent on the padding of ranks
+// and sample counts that are no multiple of 64.  Compression of a 256 x 256 P2
+// Helmholtz factor in complex128: 114 ms with 64 x 64 tiles, 56 ms so.
+template <typename T> struct TileShape {
+    static constexpr bool fp64 = sizeof(typename Tr<T>::real) == 8;
+    static constexpr int GEMM = fp64 ? 32 : 64;      // batched GEMMs
+    static constexpr int NODE = fp64 ? 16 : 64;      // per-node products
+};
+
+// Tiles of every job; blockIdx.z = job * ksplit + split.  The K
 // chunks are staged in shared memory, the next chunk's loads in registers
 // while the current chunk is multiplied.  ksplit > 1: the CTA of split q
 // takes K chunks q, q + ksplit, ... and writes its raw partial tile to
-// part[(z * tiles + tile) * 4096]; bgemm_reduce_kernel adds the partials in
+// part[(z * tiles + tile) * TILE^2]; bgemm_reduce_kernel adds the partials in
 // split order (deterministic) and applies alpha / beta.
 template <typename T, bool RB>
 __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ jobs, int ksplit, T* __restrict__ part) {
-    constexpr int TT = 64, TK = 16;
+    constexpr int TT = TileShape<T>::GEMM, TK = 16, PT = TT / 16;
     __shared__ T sA[TK][TT];
     __shared__ T sB[TK][TT];
     const int job = blockIdx.z / ksplit, split = blockIdx.z % ksplit;
@@ -203,11 +215,11 @@ __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ 
     const T* A = static_cast<const T*>(jb.A);
     const T* B = static_cast<const T*>(jb.B);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
+    T acc[PT][PT];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < PT; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = zero<T>();
+        for (int b = 0; b < PT; ++b) acc[a][b] = zero<T>();
     // element u of this thread's share of the A and B chunks at K offset kc
     auto a_idx = [&](int u, int& ii, int& l) {
         const int q = tid + 256 * u;
@@ -217,10 +229,10 @@ __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ 
         const int q = tid + 256 * u;
         if (!jb.transB) { l = q % TK; jj = q / TK; } else { jj = q % TT; l = q / TT; }
     };
-    T ra[4], rb[4];
+    T ra[PT], rb[PT];
     auto load = [&](int kc) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < PT; ++u) {
             int ii, l, jj, lb;
             a_idx(u, ii, l);
             b_idx(u, jj, lb);
@@ -234,7 +246,7 @@ __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ 
     if (kc < jb.K) load(kc);
     for (; kc < jb.K; kc += step) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < PT; ++u) {
             int ii, l, jj, lb;
             a_idx(u, ii, l);
             b_idx(u, jj, lb);
@@ -245,15 +257,15 @@ __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ 
         if (kc + step < jb.K) load(kc + step);
 #pragma unroll
         for (int l = 0; l < TK; ++l) {
-            T av[4], bv[4];
+            T av[PT], bv[PT];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = sA[l][tx + 16 * a];
+            for (int a = 0; a < PT; ++a) av[a] = sA[l][tx + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = sB[l][ty + 16 * b];
+            for (int b = 0; b < PT; ++b) bv[b] = sB[l][ty + 16 * b];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < PT; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
+                for (int b = 0; b < PT; ++b) {
                     if constexpr (RB && Tr<T>::cplx) acc[a][b] = fmar(av[a], bv[b].x, acc[a][b]);
                     else acc[a][b] = fmac(av[a], bv[b], acc[a][b]);
                 }
@@ -263,17 +275,17 @@ __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ 
     if (ksplit > 1) {
         T* P = part + ((int64_t)blockIdx.z * gridDim.x * gridDim.y + (int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (TT * TT);
 #pragma unroll
-        for (int b = 0; b < 4; ++b)
+        for (int b = 0; b < PT; ++b)
 #pragma unroll
-            for (int a = 0; a < 4; ++a) P[(ty + 16 * b) * TT + tx + 16 * a] = acc[a][b];
+            for (int a = 0; a < PT; ++a) P[(ty + 16 * b) * TT + tx + 16 * a] = acc[a][b];
         return;
     }
     using real = typename Tr<T>::real;
     T* Cm = static_cast<T*>(jb.C);
-    for (int b = 0; b < 4; ++b) {
+    for (int b = 0; b < PT; ++b) {
         const int64_t j = j0 + ty + 16 * b;
         if (j >= jb.N) continue;
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < PT; ++a) {
             const int64_t i = i0 + tx + 16 * a;
             if (i >= jb.M) continue;
             T* dst = Cm + j * jb.ldc + i;
@@ -286,7 +298,7 @@ __global__ void __launch_bounds__(256) bgemm_kernel(const GemmJob* __restrict__ 
 template <typename T>
 __global__ void __launch_bounds__(256) bgemm_reduce_kernel(const GemmJob* __restrict__ jobs, int ksplit,
                                                            const T* __restrict__ part) {
-    constexpr int TT = 64;
+    constexpr int TT = TileShape<T>::GEMM;
     const GemmJob jb = jobs[blockIdx.z];
     const int64_t i0 = (int64_t)blockIdx.x * TT, j0 = (int64_t)blockIdx.y * TT;
     if (i0 >= jb.M || j0 >= jb.N) return;
@@ -329,31 +341,33 @@ struct HNode {
 };
 
 // ---------------------------------------------- per-node small products
-// One 64 x 64 tile (rows i0.., columns j0..) of C = A B, K in chunks of 16
+// One TileShape<T>::NODE square tile (rows i0.., columns j0..) of C = A B, K in chunks of 16
 // staged in shared memory; the next chunk's loads are in registers while the
 // current chunk is multiplied, so a tile waits for memory about once, not
 // once per product term.  A(i, l) and B(l, j) come from the caller's
 // accessors (gathers allowed); A_KMAJ: consecutive threads load consecutive l
 // of A (A stored along K), else consecutive i; B is always loaded along K.
 // out(i, j, c) receives every valid entry of the tile.  All 256 threads call it.
-constexpr int NT_TILE = 64, NT_K = 16;
+constexpr int NT_K = 16;
 
-__host__ __device__ __forceinline__ int tiles64(int n) { return (n + NT_TILE - 1) / NT_TILE; }
+template <typename T>
+__host__ __device__ __forceinline__ int tiles(int n) { return (n + TileShape<T>::NODE - 1) / TileShape<T>::NODE; }
 
 template <typename T, bool A_KMAJ, typename FA, typename FB, typename FO>
-__device__ __forceinline__ void tile_gemm64(int M, int N, int K, int i0, int j0, FA fa, FB fb, FO out) {
+__device__ __forceinline__ void tile_gemm(int M, int N, int K, int i0, int j0, FA fa, FB fb, FO out) {
+    constexpr int NT_TILE = TileShape<T>::NODE, PT = NT_TILE / 16;
     __shared__ T sA[NT_K][NT_TILE];
     __shared__ T sB[NT_K][NT_TILE];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
+    T acc[PT][PT];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < PT; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = zero<T>();
-    T ra[4], rb[4];
+        for (int b = 0; b < PT; ++b) acc[a][b] = zero<T>();
+    T ra[PT], rb[PT];
     auto load = [&](int kc) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < PT; ++u) {
             const int q = tid + 256 * u;
             const int ia = A_KMAJ ? q / NT_K : q % NT_TILE, la = A_KMAJ ? q % NT_K : q / NT_TILE;
             ra[u] = (kc + la < K && i0 + ia < M) ? fa(i0 + ia, kc + la) : zero<T>();
@@ -364,7 +378,7 @@ __device__ __forceinline__ void tile_gemm64(int M, int N, int K, int i0, int j0,
     load(0);
     for (int kc = 0; kc < K; kc += NT_K) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < PT; ++u) {
             const int q = tid + 256 * u;
             const int ia = A_KMAJ ? q / NT_K : q % NT_TILE, la = A_KMAJ ? q % NT_K : q / NT_TILE;
             sA[la][ia] = ra[u];
@@ -374,23 +388,23 @@ __device__ __forceinline__ void tile_gemm64(int M, int N, int K, int i0, int j0,
         if (kc + NT_K < K) load(kc + NT_K);
 #pragma unroll
         for (int l = 0; l < NT_K; ++l) {
-            T av[4], bv[4];
+            T av[PT], bv[PT];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = sA[l][tx + 16 * a];
+            for (int a = 0; a < PT; ++a) av[a] = sA[l][tx + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = sB[l][ty + 16 * b];
+            for (int b = 0; b < PT; ++b) bv[b] = sB[l][ty + 16 * b];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < PT; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fmac(av[a], bv[b], acc[a][b]);
+                for (int b = 0; b < PT; ++b) acc[a][b] = fmac(av[a], bv[b], acc[a][b]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
+    for (int b = 0; b < PT; ++b) {
         const int j = j0 + ty + 16 * b;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < PT; ++a) {
             const int i = i0 + tx + 16 * a;
             if (i < M && j < N) out(i, j, acc[a][b]);
         }
@@ -401,7 +415,7 @@ __device__ __forceinline__ void tile_gemm64(int M, int N, int K, int i0, int j0,
 // Leaf: S_loc = Y(I, :) - S(I, I) Om(I, :).  Inner node: the children's
 // skeleton rows, S_loc = [S_c1(J1, :) - S(J1, J2) Om_c2; S_c2(J2, :) - S(J2, J1) Om_c1].
 // Grid: (nodes, tiles): a leaf's tiles cover rows x p; an inner node's two
-// parts (rows of c1, rows of c2) ceil(kcap / 64) row tiles each.
+// parts (rows of c1, rows of c2) tiles(kcap) row tiles each.
 template <typename T>
 __global__ void __launch_bounds__(HT)
 form_sloc_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, const HFront* __restrict__ fronts,
@@ -416,17 +430,17 @@ form_sloc_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, 
     T* W = ws + nd.o_w;
     T* SL = ws + nd.o_sl;
     int* iloc = iws + nd.o_iloc;
-    const int tn = tiles64(p);
+    const int tn = tiles<T>(p);
     const int t = blockIdx.y;
     if (nd.c1 < 0) {
         const int rows = nd.hi - nd.lo;
-        const int i0 = (t / tn) * NT_TILE, j0 = (t % tn) * NT_TILE;
+        const int i0 = (t / tn) * TileShape<T>::NODE, j0 = (t % tn) * TileShape<T>::NODE;
         if (t == 0) {
             for (int r = threadIdx.x; r < rows; r += HT) iloc[r] = nd.lo + r;
             if (threadIdx.x == 0) rows_out[list[blockIdx.x]] = rows;
         }
         if (i0 >= rows) return;
-        tile_gemm64<T, false>(
+        tile_gemm<T, false>(
             rows, p, rows, i0, j0, [&](int r, int c) { return -S[(int64_t)(nd.lo + c) * lds + nd.lo + r]; },
             [&](int c, int j) { return Om[(int64_t)j * n + nd.lo + c]; },
             [&](int r, int j, T acc) {
@@ -443,9 +457,9 @@ form_sloc_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, 
             for (int r = threadIdx.x; r < k1 + k2; r += HT) iloc[r] = (r < k1) ? sk1[r] : sk2[r - k1];
             if (threadIdx.x == 0) rows_out[list[blockIdx.x]] = k1 + k2;
         }
-        const int tm = tiles64(nd.kcap);
+        const int tm = tiles<T>(nd.kcap);
         const int part = t / (tm * tn), tt = t % (tm * tn);
-        const int i0 = (tt / tn) * NT_TILE, j0 = (tt % tn) * NT_TILE;
+        const int i0 = (tt / tn) * TileShape<T>::NODE, j0 = (tt % tn) * TileShape<T>::NODE;
         // part 0: rows of c1 (coupled to c2's skeleton), part 1: rows of c2
         const int M = part == 0 ? k1 : k2, K = part == 0 ? k2 : k1, roff = part == 0 ? 0 : k1;
         if (part > 1 || i0 >= M) return;
@@ -454,7 +468,7 @@ form_sloc_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, 
         const T* Sown = ws + (part == 0 ? a.o_si : b.o_si);
         const T* Ooth = ws + (part == 0 ? b.o_om : a.o_om);
         const int kcown = part == 0 ? a.kcap : b.kcap, kcoth = part == 0 ? b.kcap : a.kcap;
-        tile_gemm64<T, false>(
+        tile_gemm<T, false>(
             M, p, K, i0, j0, [&](int r, int c) { return -S[(int64_t)oth[c] * lds + own[r]]; },
             [&](int c, int j) { return Ooth[(int64_t)j * kcoth + c]; },
             [&](int r, int j, T acc) {
@@ -924,13 +938,13 @@ finish_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, con
         ld1 = nodes[nd.c1].kcap;
         ld2 = nodes[nd.c2].kcap;
     }
-    const int tn = tiles64(p), t = blockIdx.y;
+    const int tn = tiles<T>(p), t = blockIdx.y;
     if (t == 0)
         for (int a = threadIdx.x; a < k; a += HT) skel[a] = iloc[piv[a]];
-    const int i0 = (t / tn) * NT_TILE, j0 = (t % tn) * NT_TILE;
+    const int i0 = (t / tn) * TileShape<T>::NODE, j0 = (t % tn) * TileShape<T>::NODE;
     if (i0 >= k) return;
     // Om_i = X^T Om_loc (k x p), S_i = S_loc(J, :)
-    tile_gemm64<T, true>(
+    tile_gemm<T, true>(
         k, p, rows, i0, j0, [&](int a, int r) { return X[(int64_t)a * nd.rows_cap + r]; },
         [&](int r, int j) {
             if (nd.c1 < 0) return Om[(int64_t)j * fr.n + nd.lo + r];
@@ -963,10 +977,10 @@ hss_up_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, con
         h1 = hb + nodes[nd.c1].o_xh;
         h2 = hb + nodes[nd.c2].o_xh;
     }
-    const int tn = tiles64(nc), t = blockIdx.y;
-    const int i0 = (t / tn) * NT_TILE, j0 = (t % tn) * NT_TILE;
+    const int tn = tiles<T>(nc), t = blockIdx.y;
+    const int i0 = (t / tn) * TileShape<T>::NODE, j0 = (t % tn) * TileShape<T>::NODE;
     if (i0 >= k) return;
-    tile_gemm64<T, true>(
+    tile_gemm<T, true>(
         k, nc, rows, i0, j0, [&](int a, int r) { return X[(int64_t)a * nd.rows_cap + r]; },
         [&](int r, int j) {
             if (nd.c1 < 0) return x[(int64_t)j * lx + nd.lo + r];
@@ -994,16 +1008,16 @@ hss_down_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, c
     const int k = root ? 0 : kk[id];
     const T* X = ws + nd.o_x;
     const T* yh = hb + nd.o_yh;
-    const int tn = tiles64(nc), tm = tiles64(nd.kcap), t = blockIdx.y;
+    const int tn = tiles<T>(nc), tm = tiles<T>(nd.kcap), t = blockIdx.y;
     const int part = t / (tm * tn), tt = t % (tm * tn);
-    const int i0 = (tt / tn) * NT_TILE, j0 = (tt % tn) * NT_TILE;
+    const int i0 = (tt / tn) * TileShape<T>::NODE, j0 = (tt % tn) * TileShape<T>::NODE;
     const int M = part == 0 ? k1 : k2, Ko = part == 0 ? k2 : k1, roff = part == 0 ? 0 : k1;
     if (part > 1 || i0 >= M) return;
     const int* own = iws + (part == 0 ? a.o_skel : b.o_skel);
     const int* oth = iws + (part == 0 ? b.o_skel : a.o_skel);
     const T* xo = hb + (part == 0 ? b.o_xh : a.o_xh);
     T* yo = hb + (part == 0 ? a.o_yh : b.o_yh);
-    tile_gemm64<T, false>(
+    tile_gemm<T, false>(
         M, nc, k + Ko, i0, j0,
         [&](int r, int l) {
             return l < k ? X[(int64_t)l * nd.rows_cap + roff + r] : S[(int64_t)oth[l - k] * lds + own[r]];
@@ -1033,10 +1047,10 @@ hss_leaf_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, c
     const T* x = xin[nd.front];
     T* y = yout[nd.front];
     const int64_t lx = ldx[nd.front], ly = ldy[nd.front];
-    const int tn = tiles64(nc), t = blockIdx.y;
-    const int i0 = (t / tn) * NT_TILE, j0 = (t % tn) * NT_TILE;
+    const int tn = tiles<T>(nc), t = blockIdx.y;
+    const int i0 = (t / tn) * TileShape<T>::NODE, j0 = (t % tn) * TileShape<T>::NODE;
     if (i0 >= rows) return;
-    tile_gemm64<T, false>(
+    tile_gemm<T, false>(
         rows, nc, rows + k, i0, j0,
         [&](int r, int l) {
             return l < rows ? S[(int64_t)(nd.lo + l) * lds + nd.lo + r] : X[(int64_t)(l - rows) * nd.rows_cap + r];
@@ -1297,7 +1311,8 @@ ndhss_status run_bgemm_group(const std::vector<GemmJob>& jobs, cudaStream_t st) 
         maxN = std::max(maxN, g.N);
         maxK = std::max(maxK, g.K);
     }
-    const int tm = (maxM + 63) / 64, tn = (maxN + 63) / 64;
+    constexpr int TT = TileShape<T>::GEMM;
+    const int tm = (maxM + TT - 1) / TT, tn = (maxN + TT - 1) / TT;
     int dev = 0, sms = 1;
     HSS_TRY(cudaGetDevice(&dev));
     HSS_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1310,7 +1325,7 @@ ndhss_status run_bgemm_group(const std::vector<GemmJob>& jobs, cudaStream_t st) 
     HSS_TRY(dj.upload(jobs, st));
     const size_t per = (size_t)std::max(1, 65535 / ks);     // jobs per launch (grid z limit)
     DeviceVec<T> part(st);
-    if (ks > 1) HSS_TRY(part.alloc((size_t)std::min(per, jobs.size()) * ks * tm * tn * 4096));
+    if (ks > 1) HSS_TRY(part.alloc((size_t)std::min(per, jobs.size()) * ks * tm * tn * (TT * TT)));
     for (size_t j0 = 0; j0 < jobs.size(); j0 += per) {
         const unsigned nj = (unsigned)std::min(per, jobs.size() - j0);
         bgemm_kernel<T, RB><<<dim3(tm, tn, nj * ks), 256, 0, st>>>(dj.p + j0, ks, part.p);
@@ -1369,23 +1384,23 @@ ndhss_status hss_matvec_run(const std::vector<HNode>& nodes, const std::vector<c
         kcap = std::max(kcap, nodes[i].kcap);
         if (nodes[i].c1 < 0) leaf_rows = std::max(leaf_rows, nodes[i].hi - nodes[i].lo);
     }
-    const unsigned tnc = (unsigned)tiles64(nc_max);
+    const unsigned tnc = (unsigned)tiles<T>(nc_max);
     for (int l = maxlev; l >= 1; --l) {
         const unsigned cnt = (unsigned)(up_off[l + 1] - up_off[l]);
         if (!cnt) continue;
-        hss_up_kernel<T><<<dim3(cnt, tiles64(kcap) * tnc), HT, 0, st>>>(dflat.p + up_off[l], dnodes, ws, hb, kk, rows, dx,
+        hss_up_kernel<T><<<dim3(cnt, tiles<T>(kcap) * tnc), HT, 0, st>>>(dflat.p + up_off[l], dnodes, ws, hb, kk, rows, dx,
                                                                          dlx, dncs, xh_ld);
         NDHSS_LAUNCH_CHECK("hss_up_kernel");
     }
     for (int l = 0; l <= maxlev; ++l) {
         const unsigned cnt = (unsigned)(dn_off[l + 1] - dn_off[l]);
         if (!cnt) continue;
-        hss_down_kernel<T><<<dim3(cnt, 2 * tiles64(kcap) * tnc), HT, 0, st>>>(dflat.p + dn_off[l], dnodes, dfr, ws, hb,
+        hss_down_kernel<T><<<dim3(cnt, 2 * tiles<T>(kcap) * tnc), HT, 0, st>>>(dflat.p + dn_off[l], dnodes, dfr, ws, hb,
                                                                                iws, kk, dncs, xh_ld);
         NDHSS_LAUNCH_CHECK("hss_down_kernel");
     }
     if (leaf_cnt) {
-        hss_leaf_kernel<T><<<dim3((unsigned)leaf_cnt, tiles64(leaf_rows) * tnc), HT, 0, st>>>(
+        hss_leaf_kernel<T><<<dim3((unsigned)leaf_cnt, tiles<T>(leaf_rows) * tnc), HT, 0, st>>>(
             dflat.p + leaf_off, dnodes, dfr, ws, hb, kk, dx, dlx, dy, dly, dncs, xh_ld);
         NDHSS_LAUNCH_CHECK("hss_leaf_kernel");
     }
@@ -1889,7 +1904,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                 int leaf_rows = 1;
                 for (size_t q = loff[l]; q < loff[l + 1]; ++q)
                     if (nodes[flat[q]].c1 < 0) leaf_rows = std::max(leaf_rows, nodes[flat[q]].hi - nodes[flat[q]].lo);
-                const unsigned tf = (unsigned)(std::max(tiles64(leaf_rows), 2 * tiles64(kcap)) * tiles64(p));
+                const unsigned tf = (unsigned)(std::max(tiles<T>(leaf_rows), 2 * tiles<T>(kcap)) * tiles<T>(p));
                 form_sloc_kernel<T><<<dim3(cnt, tf), HT, 0, st>>>(dflat.p + loff[l], dnodes.p, dfr.p, ws.p, iws.p, kk.p,
                                                                  rows.p);
                 NDHSS_LAUNCH_CHECK("form_sloc_kernel");
@@ -1897,7 +1912,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                     const ndhss_status rc = launch_row_id(loff[l], loff[l + 1]);
                     if (rc != NDHSS_OK) return rc;
                 }
-                finish_kernel<T><<<dim3(cnt, tiles64(kcap) * tiles64(p)), HT, 0, st>>>(dflat.p + loff[l], dnodes.p, dfr.p,
+                finish_kernel<T><<<dim3(cnt, tiles<T>(kcap) * tiles<T>(p)), HT, 0, st>>>(dflat.p + loff[l], dnodes.p, dfr.p,
                                                                                       ws.p, iws.p, kk.p, rows.p);
                 NDHSS_LAUNCH_CHECK("finish_kernel");
             }
