@@ -22,6 +22,7 @@
 #include <climits>
 #include <cstdlib>
 #include <cmath>
+#include <cstring>
 #include <memory>
 #include <mutex>
 #include <type_traits>
@@ -1199,21 +1200,86 @@ std::vector<HCl> cluster_tree(int n, int top, int beta) {
 // Stream-ordered scratch (pool allocator): no device-wide synchronisation on
 // allocation or release, uploads from pageable host memory are staged by the
 // runtime before cudaMemcpyAsync returns.
+// Memory for the small host tables of one compression call on one stream: a
+// device block from the pool and a page-locked block, both handed out in
+// order.  The device block starts over with a sampling round (its copies are
+// ordered after the kernels of the round before), the page-locked one once
+// the stream has been synchronised.  What does not fit takes the ordinary way.
+// (129 x 75 P1 Helmholtz, 110 tables per factorization, a pool allocation and a
+// pageable copy each: the GPU idled 1.5 of 5.1 ms before them.)
+struct TableArena {
+    static constexpr size_t DEV_BYTES = size_t(8) << 20;
+    PinnedBuf* host = nullptr;
+    unsigned char* dev = nullptr;
+    size_t hoff = 0, doff = 0;
+    cudaStream_t st;
+    TableArena* outer;
+    static TableArena*& current() {
+        thread_local TableArena* t = nullptr;
+        return t;
+    }
+    explicit TableArena(cudaStream_t s) : st(s), outer(current()) {
+        host = pinned_acquire();
+        if (pool_malloc_async((void**)&dev, DEV_BYTES, st) != cudaSuccess) {
+            cudaGetLastError();
+            dev = nullptr;
+        }
+        current() = this;
+    }
+    TableArena(const TableArena&) = delete;
+    TableArena& operator=(const TableArena&) = delete;
+    ~TableArena() {
+        current() = outer;
+        if (dev) cudaFreeAsync(dev, st);
+        pinned_release(host, st);
+    }
+    void new_round() { doff = 0; }
+    void synchronised() { hoff = 0; }
+    // the device copy of a table, or null when it does not fit
+    void* put(const void* src, size_t bytes, cudaStream_t s) {
+        const size_t need = (bytes + 255) / 256 * 256;
+        if (s != st || !host || !dev || hoff + need > PINNED_BYTES || doff + need > DEV_BYTES) return nullptr;
+        std::memcpy(host->p + hoff, src, bytes);
+        if (cudaMemcpyAsync(dev + doff, host->p + hoff, bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        void* d = dev + doff;
+        hoff += need;
+        doff += need;
+        return d;
+    }
+};
+
 template <typename U>
 struct DeviceVec {
     U* p = nullptr;
     size_t n = 0;
     cudaStream_t st = nullptr;
+    bool owned = true;                    // false: part of the call's TableArena
     explicit DeviceVec(cudaStream_t s = nullptr) : st(s) {}
-    ~DeviceVec() { if (p) cudaFreeAsync(p, st); }
-    cudaError_t alloc(size_t count) {
-        if (p) cudaFreeAsync(p, st);
+    ~DeviceVec() { release(); }
+    void release() {
+        if (p && owned) cudaFreeAsync(p, st);
         p = nullptr;
+        owned = true;
+    }
+    cudaError_t alloc(size_t count) {
+        release();
         n = count;
         return pool_malloc_async((void**)&p, std::max<size_t>(n, 1) * sizeof(U), st);
     }
     cudaError_t upload(const std::vector<U>& v, cudaStream_t s) {
+        release();
         st = s;
+        n = v.size();
+        if (TableArena* t = v.empty() ? nullptr : TableArena::current()) {
+            p = static_cast<U*>(t->put(v.data(), v.size() * sizeof(U), st));
+            if (p) {
+                owned = false;
+                return cudaSuccess;
+            }
+        }
         cudaError_t e = alloc(v.size());
         if (e == cudaSuccess && !v.empty()) e = cudaMemcpyAsync(p, v.data(), v.size() * sizeof(U), cudaMemcpyHostToDevice, st);
         return e;
@@ -1605,7 +1671,9 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
     std::vector<double> prev_err(probs.size(), INFINITY);
     int p = k0 + r;
     int round = 0;
+    TableArena tables(st);
     while (!active.empty()) {
+        tables.new_round();
         const int kcap = std::max(1, std::min(rank_cap, p - OVERSAMPLE_MIN));
         std::vector<HFront> fr;
         std::vector<HNode> nodes;
@@ -1949,6 +2017,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
         HSS_TRY(cudaMemcpyAsync(hn.data(), dn.p, hn.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
         HSS_TRY(cudaMemcpyAsync(hk.data(), kk.p, hk.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
         HSS_TRY(cudaStreamSynchronize(st));
+        tables.synchronised();
         std::vector<int> done, still;
         for (int i = 0; i < nf; ++i) {
             const Problem& pb = probs[active[i]];

@@ -5,10 +5,21 @@
 // remapping ~100 MB of GMRES work space costs far more than the solve step
 // it serves).  The pool is created on first use per device and lives until
 // the process exits.
+//
+// Page-locked staging buffers for small host tables: a copy from pageable
+// memory costs the host several microseconds each, and the compression's
+// rounds upload a dozen tables per round.  A buffer belongs to one call at a
+// time; it is handed out again once the copies of the call before have run
+// (an event on that call's stream).  At most PINNED_KEEP free buffers per
+// process are kept.
 #include <cstdint>
 #include <mutex>
+#include <new>
+#include <vector>
 
 #include <cuda_runtime.h>
+
+#include "mempool.h"
 
 namespace ndhss {
 
@@ -46,6 +57,66 @@ cudaError_t pool_malloc_async(void** p, size_t bytes, cudaStream_t st) {
         pool = g_pool[dev];
     }
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
+namespace {
+constexpr size_t PINNED_KEEP = 4;
+std::mutex g_pinned_mu;
+std::vector<PinnedBuf*>& pinned_free() {
+    static std::vector<PinnedBuf*>* v = new std::vector<PinnedBuf*>();     // lives until the process exits
+    return *v;
+}
+void pinned_destroy(PinnedBuf* b) {
+    if (b->p) cudaFreeHost(b->p);
+    if (b->ev) cudaEventDestroy(b->ev);
+    delete b;
+}
+}  // namespace
+
+PinnedBuf* pinned_acquire() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    PinnedBuf* b = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_pinned_mu);
+        std::vector<PinnedBuf*>& v = pinned_free();
+        for (size_t i = v.size(); i-- > 0 && !b;)
+            if (v[i]->dev == dev) {
+                b = v[i];
+                v.erase(v.begin() + (std::ptrdiff_t)i);
+            }
+    }
+    if (b) {
+        if (cudaEventSynchronize(b->ev) == cudaSuccess) return b;
+        cudaGetLastError();
+        pinned_destroy(b);
+        return nullptr;
+    }
+    b = new (std::nothrow) PinnedBuf();
+    if (!b) return nullptr;
+    b->dev = dev;
+    if (cudaHostAlloc(reinterpret_cast<void**>(&b->p), PINNED_BYTES, cudaHostAllocDefault) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        pinned_destroy(b);
+        return nullptr;
+    }
+    return b;
+}
+
+void pinned_release(PinnedBuf* b, cudaStream_t st) {
+    if (!b) return;
+    bool keep = cudaEventRecord(b->ev, st) == cudaSuccess;
+    if (keep) {
+        std::lock_guard<std::mutex> lock(g_pinned_mu);
+        keep = pinned_free().size() < PINNED_KEEP;
+        if (keep) pinned_free().push_back(b);
+    }
+    if (!keep) {
+        cudaStreamSynchronize(st);
+        cudaGetLastError();
+        pinned_destroy(b);
+    }
 }
 
 }  // namespace ndhss
