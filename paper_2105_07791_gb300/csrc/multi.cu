@@ -39,8 +39,16 @@ constexpr int MR = 32;            // interleaved right-hand sides
 constexpr int MT_ROWS = 64;       // rows per apply tile
 constexpr int MT_K = 16;          // K chunk of an apply tile
 constexpr int MT_THREADS = 128;   // threads of a dense apply tile (4 x 4 products each)
+constexpr int MT_DEEP = 4 * 152;  // levels with fewer 32-row tiles split K over four groups
 constexpr int MF_ROWS = 8, MF_COLS = 4, MF_THREADS = 128;   // FP64 apply: outputs per CTA, four warps over K
 constexpr int SEG_ROWS = 1024;    // rows per reduction block
+// The row-wise kernels (product, vector updates) split a reduction block over
+// SEG_PARTS CTAs: 16 problems make about 400 blocks, under three CTAs per SM,
+// too few warps to wait for memory with (product of 16 uneven P1 Helmholtz
+// problems x 32 columns: 0.82 ms with one CTA per block and four DFMA per
+// entry, 0.56 so).
+constexpr int SEG_PARTS = 4;
+constexpr int DOT_WARPS = 16;     // warps of a dot-product block
 constexpr int BK = 32;            // restart + 1 <= BK
 
 __device__ __forceinline__ double babs(double a) { return fabs(a); }
@@ -91,15 +99,29 @@ __global__ void mscatter_kernel(int64_t n, int nrhs, const int32_t* __restrict__
 // UP = the first m_i columns of the front against u(I^s o sigma) (rows < m_i
 // to z, rows >= m_i subtracted from u(B^s)); !UP = the R block against
 // z(B^s), added to z(I^s).
-template <typename T, bool UP, int ROWS>
-__global__ void __launch_bounds__(2 * ROWS)
+//
+// KG groups of 2 ROWS threads share the K chunks (group g takes chunks g,
+// g + KG, ...) and add their sums in group order.  KG = 4 on the levels whose
+// tiles leave the SMs without warps (MT_DEEP): a root of 250 unknowns is a
+// chain of 16 chunks, each a memory wait and two barriers, in 60 CTAs of two
+// warps.  Eight P1 Helmholtz problems x 32 columns: 55 us for the root level
+// with one group.
+template <typename T, bool UP, int ROWS, int KG>
+__global__ void __launch_bounds__(2 * ROWS * KG)
 mapply_kernel(const int2* __restrict__ jobs, const int32_t* __restrict__ node, const int64_t* __restrict__ foff,
               const T* __restrict__ front, const int32_t* __restrict__ sigma, const int32_t* __restrict__ blist,
               T* __restrict__ U, T* __restrict__ Z, const int* __restrict__ pact, const int32_t* __restrict__ nprob,
               const uint64_t* __restrict__ lr_ptr) {
     constexpr int NTH = 2 * ROWS;
-    __shared__ __align__(16) T As[MT_K][ROWS];
-    __shared__ __align__(16) T Bs[MT_K][MR];
+    __shared__ __align__(16) T sm[KG * MT_K * (ROWS + MR)];
+    const int grp = threadIdx.x / NTH;
+    T (*As)[ROWS] = reinterpret_cast<T(*)[ROWS]>(sm + grp * MT_K * ROWS);
+    T (*Bs)[MR] = reinterpret_cast<T(*)[MR]>(sm + KG * MT_K * ROWS + grp * MT_K * MR);
+    // the group's barrier
+    auto sync = [&]() {
+        if constexpr (KG == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(NTH) : "memory");
+    };
     const int2 J = jobs[blockIdx.x];
     const int s = J.x, r0 = J.y;
     if (pact && !pact[nprob[s]]) return;          // a problem whose systems all stopped
@@ -115,7 +137,7 @@ mapply_kernel(const int2* __restrict__ jobs, const int32_t* __restrict__ node, c
     const T* src = UP ? U : Z;
     // thread (ty, tx) owns rows 4 ty .. 4 ty + 3 and columns 4 tx .. 4 tx + 3
     // of the tile (16 products per 64 bytes read from shared memory)
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int tid = threadIdx.x % NTH, tx = tid & 7, ty = tid >> 3;
     T acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -143,11 +165,11 @@ mapply_kernel(const int2* __restrict__ jobs, const int32_t* __restrict__ node, c
             rb[u] = sr >= 0 ? src[(int64_t)sr * MR + c] : zero<T>();
         }
     };
-    if (K > 0) {
-        load_a(0);
-        load_b(0);
+    if (grp * MT_K < K) {
+        load_a(grp * MT_K);
+        load_b(grp * MT_K);
     }
-    for (int k0 = 0; k0 < K; k0 += MT_K) {
+    for (int k0 = grp * MT_K; k0 < K; k0 += KG * MT_K) {
 #pragma unroll
         for (int u = 0; u < ROWS * MT_K / NTH; ++u) {
             const int q = tid + NTH * u;
@@ -158,10 +180,10 @@ mapply_kernel(const int2* __restrict__ jobs, const int32_t* __restrict__ node, c
             const int q = tid + NTH * u;
             Bs[q / MR][q % MR] = rb[u];
         }
-        __syncthreads();
-        if (k0 + MT_K < K) {
-            load_a(k0 + MT_K);
-            load_b(k0 + MT_K);
+        sync();
+        if (k0 + KG * MT_K < K) {
+            load_a(k0 + KG * MT_K);
+            load_b(k0 + KG * MT_K);
         }
 #pragma unroll
         for (int kk = 0; kk < MT_K; ++kk) {
@@ -175,7 +197,20 @@ mapply_kernel(const int2* __restrict__ jobs, const int32_t* __restrict__ node, c
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmac(a[i], bv[j], acc[i][j]);
         }
+        sync();
+    }
+    if constexpr (KG > 1) {
+        static_assert((KG - 1) * NTH * 16 <= KG * MT_K * (ROWS + MR), "the groups' sums fit the operand buffers");
         __syncthreads();
+        if (grp > 0)
+#pragma unroll
+            for (int q = 0; q < 16; ++q) sm[((grp - 1) * 16 + q) * NTH + tid] = acc[q / 4][q % 4];
+        __syncthreads();
+        if (grp > 0) return;
+#pragma unroll
+        for (int g = 0; g < KG - 1; ++g)
+#pragma unroll
+            for (int q = 0; q < 16; ++q) acc[q / 4][q % 4] = acc[q / 4][q % 4] + sm[(g * 16 + q) * NTH + tid];
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -428,14 +463,16 @@ ndhss_status multi_apply_run(const FactorData& F, int nrhs, const V* X, int64_t 
                     mapply_fp64_kernel<T, true><<<grid, MF_THREADS, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
                 else
                     mapply_fp64_kernel<T, false><<<grid, MF_THREADS, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
-            } else if (up && v == 0)
-                mapply_kernel<T, true, 32><<<(unsigned)(b - a), 64, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
-            else if (up)
-                mapply_kernel<T, true, 64><<<(unsigned)(b - a), 128, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
-            else if (v == 0)
-                mapply_kernel<T, false, 32><<<(unsigned)(b - a), 64, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
-            else
-                mapply_kernel<T, false, 64><<<(unsigned)(b - a), 128, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
+            } else {
+                const bool deep = (up ? F.mj_up_tiles : F.mj_dn_tiles)[l] < MT_DEEP;
+                auto launch = [&](auto kernel, int threads) {
+                    kernel<<<(unsigned)(b - a), threads, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
+                };
+                if (up && v == 0) deep ? launch(mapply_kernel<T, true, 32, 4>, 256) : launch(mapply_kernel<T, true, 32, 1>, 64);
+                else if (up) deep ? launch(mapply_kernel<T, true, 64, 4>, 512) : launch(mapply_kernel<T, true, 64, 1>, 128);
+                else if (v == 0) deep ? launch(mapply_kernel<T, false, 32, 4>, 256) : launch(mapply_kernel<T, false, 32, 1>, 64);
+                else deep ? launch(mapply_kernel<T, false, 64, 4>, 512) : launch(mapply_kernel<T, false, 64, 1>, 128);
+            }
             NDHSS_LAUNCH_CHECK("mapply_kernel");
         }
         return NDHSS_OK;
@@ -497,6 +534,11 @@ ndhss_status multi_supported(const FactorData& F, const char* who) {
 struct Seg {
     int32_t s, row0, row1, pad;
 };
+// this CTA's part of its block (blockIdx.y of SEG_PARTS)
+__device__ __forceinline__ void seg_part(Seg& g) {
+    g.row0 += (int)blockIdx.y * (SEG_ROWS / SEG_PARTS);
+    g.row1 = min(g.row1, g.row0 + SEG_ROWS / SEG_PARTS);
+}
 
 enum : int32_t { ST_ACTIVE = 0, ST_STOPPED = 1, ST_CONVERGED = 2, ST_FAILED = 3, ST_PAD = 4 };
 
@@ -507,38 +549,92 @@ struct BState {
     int32_t status, jend, its, cycles;
 };
 
+// NP products of one row's entries (the same in every lane) with the lanes'
+// columns; the imaginary parts only when the batch holds one
+__device__ __forceinline__ bool has_imag(double) { return false; }
+__device__ __forceinline__ bool has_imag(c128 a) { return __double_as_longlong(a.y) << 1 != 0; }
+template <int NP>
+__device__ __forceinline__ void spmm_fmas(const double* a, const double* xv, double& acc, bool) {
+#pragma unroll
+    for (int u = 0; u < NP; ++u) acc = fma(a[u], xv[u], acc);
+}
+template <int NP>
+__device__ __forceinline__ void spmm_fmas(const c128* a, const c128* xv, c128& acc, bool any_imag) {
+#pragma unroll
+    for (int u = 0; u < NP; ++u) {
+        acc.x = fma(a[u].x, xv[u].x, acc.x);
+        acc.y = fma(a[u].x, xv[u].y, acc.y);
+    }
+    if (any_imag) {
+#pragma unroll
+        for (int u = 0; u < NP; ++u) {
+            acc.x = fma(-a[u].y, xv[u].y, acc.x);
+            acc.y = fma(a[u].y, xv[u].x, acc.y);
+        }
+    }
+}
+
 // Y(:, c) = A X(:, c) for the 32 interleaved columns of one block of rows
 // per CTA: one warp per row, lane = column; blocks of a problem with
-// pact[s] == 0 are skipped (pact null: every block)
+// pact[s] == 0 are skipped (pact null: every block).  Up to eight
+// entries are loaded together, then exactly their products are issued (a
+// predicated-off DFMA costs as much as one that runs), the imaginary parts only
+// when an entry of the batch holds one (the impedance term sits on the
+// boundary); the vote makes that a branch.
 template <typename V>
 __global__ void __launch_bounds__(256)
 spmm_kernel(const Seg* __restrict__ segs, const int* __restrict__ pact, const int32_t* __restrict__ rowptr,
             const int32_t* __restrict__ col, const V* __restrict__ vals, const V* __restrict__ X, V* __restrict__ Y) {
-    const Seg sg = segs[blockIdx.x];
+    constexpr int U = 8;
+    Seg sg = segs[blockIdx.x];
     if (pact && !pact[sg.s]) return;
+    seg_part(sg);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int row = sg.row0 + warp; row < sg.row1; row += 8) {
         V acc = zero<V>();
-        for (int k = rowptr[row]; k < rowptr[row + 1]; ++k) acc = fmac(vals[k], X[(int64_t)col[k] * MR + lane], acc);
+        const int k1 = rowptr[row + 1];
+        for (int k = rowptr[row]; k < k1; k += U) {
+            const int np = min(U, k1 - k);
+            int c[U];
+            V a[U], xv[U];
+            bool im = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                c[u] = u < np ? col[k + u] : -1;
+                a[u] = u < np ? vals[k + u] : zero<V>();
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                xv[u] = c[u] >= 0 ? X[(int64_t)c[u] * MR + lane] : zero<V>();
+                im = im || has_imag(a[u]);
+            }
+            im = __any_sync(0xffffffffu, im);
+            switch (np) {
+#define NDHSS_SPM(NN) case NN: spmm_fmas<NN>(a, xv, acc, im); break;
+                NDHSS_SPM(1) NDHSS_SPM(2) NDHSS_SPM(3) NDHSS_SPM(4) NDHSS_SPM(5) NDHSS_SPM(6) NDHSS_SPM(7) NDHSS_SPM(8)
+#undef NDHSS_SPM
+                default: break;
+            }
+        }
         Y[(int64_t)row * MR + lane] = acc;
     }
 }
 
 // part[blk][i][c] = sum over the block's rows of conj(V_i(row, c)) w(row, c),
-// i < nvec.  Lane = column, warp = a contiguous eighth of the block's rows,
+// i < nvec.  Lane = column, warp = a contiguous part of the block's rows,
 // four basis vectors per pass and four rows per iteration, so every warp has
 // 4 + 16 independent 512-byte loads in flight (the float64 accumulation
 // chains are too slow to wait on one load at a time).
 template <typename V>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(32 * DOT_WARPS, 2)
 bdot_kernel(const Seg* __restrict__ segs, const int* __restrict__ pact, const V* __restrict__ Vb, int64_t ldv, int nvec,
             const V* __restrict__ w, V* __restrict__ part) {
     constexpr int NB = 4, UR = 4;
-    __shared__ V red[NB][8][MR];
+    __shared__ V red[NB][DOT_WARPS][MR];
     const Seg sg = segs[blockIdx.x];
     if (pact && !pact[sg.s]) return;
     const int c = threadIdx.x & 31, rg = threadIdx.x >> 5;
-    const int len = sg.row1 - sg.row0, per = (len + 7) / 8;
+    const int len = sg.row1 - sg.row0, per = (len + DOT_WARPS - 1) / DOT_WARPS;
     const int r0 = sg.row0 + rg * per, r1 = min(sg.row1, r0 + per);
     for (int i0 = 0; i0 < nvec; i0 += NB) {
         const int ni = min(NB, nvec - i0);
@@ -574,7 +670,7 @@ bdot_kernel(const Seg* __restrict__ segs, const int* __restrict__ pact, const V*
         for (int q = threadIdx.x; q < ni * MR; q += blockDim.x) {
             const int ii = q / MR, cc = q % MR;
             V sum = red[ii][0][cc];
-            for (int g = 1; g < 8; ++g) sum = sum + red[ii][g][cc];
+            for (int g = 1; g < DOT_WARPS; ++g) sum = sum + red[ii][g][cc];
             part[((int64_t)blockIdx.x * BK + i0 + ii) * MR + cc] = sum;
         }
         __syncthreads();
@@ -603,8 +699,9 @@ baxpy_kernel(const Seg* __restrict__ segs, const int* __restrict__ pact, int nsy
              int64_t ldv, int nvec, const V* __restrict__ h, double sign, V* __restrict__ w,
              const BState* __restrict__ bs) {
     __shared__ V sh[BK][MR];
-    const Seg sg = segs[blockIdx.x];
+    Seg sg = segs[blockIdx.x];
     if (pact && !pact[sg.s]) return;
+    seg_part(sg);
     const int Q = nsys * MR;
     for (int q = threadIdx.x; q < nvec * MR; q += blockDim.x) sh[q / MR][q % MR] = h[(int64_t)(q / MR) * Q + sg.s * MR + q % MR];
     __syncthreads();
@@ -626,8 +723,9 @@ baxpy_kernel(const Seg* __restrict__ segs, const int* __restrict__ pact, int nsy
 template <typename V>
 __global__ void bscale_kernel(const Seg* __restrict__ segs, const int* __restrict__ pact, const BState* __restrict__ bs,
                               const V* __restrict__ src, V* __restrict__ dst) {
-    const Seg sg = segs[blockIdx.x];
+    Seg sg = segs[blockIdx.x];
     if (pact && !pact[sg.s]) return;
+    seg_part(sg);
     const int c = threadIdx.x & 31, rg = threadIdx.x >> 5;
     const double f = bs[sg.s * MR + c].inv;
     for (int row = sg.row0 + rg; row < sg.row1; row += 8) {
@@ -886,8 +984,9 @@ ndhss_status gmres_batched_run(const FactorData& F, const int32_t* rowptr, const
     const int qb = (Q + 255) / 256;
     binterleave_kernel<V><<<eb, 256, 0, st>>>(n, nrhs, b, ldb, Bi);
     NDHSS_LAUNCH_CHECK("binterleave_kernel");
+    const dim3 seg_grid((unsigned)nseg, SEG_PARTS);
     auto dots = [&](const V* basis, int nvec, const V* vec, V* out, const int* mask) {
-        bdot_kernel<V><<<nseg, 256, 0, st>>>(d_seg, mask, basis, nm, nvec, vec, part);
+        bdot_kernel<V><<<nseg, 32 * DOT_WARPS, 0, st>>>(d_seg, mask, basis, nm, nvec, vec, part);
         breduce_kernel<V><<<(Q * nvec + 255) / 256, 256, 0, st>>>(nsys, d_soff, nvec, part, out);
     };
     auto read_count = [&](int* h) -> ndhss_status {
@@ -900,7 +999,7 @@ ndhss_status gmres_batched_run(const FactorData& F, const int32_t* rowptr, const
     binit_kernel<V><<<qb, 256, 0, st>>>(Q, nrhs, n2, o.cycle_rtol, bs);
     NDHSS_LAUNCH_CHECK("binit_kernel");
     while (true) {
-        spmm_kernel<V><<<nseg, 256, 0, st>>>(d_seg, nullptr, rowptr, col, vals, Xi, t);
+        spmm_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, nullptr, rowptr, col, vals, Xi, t);
         ++nspmv;
         bsub_kernel<V><<<eb, 256, 0, st>>>(nm, Bi, t, w);
         dots(w, 1, w, n2, nullptr);
@@ -915,30 +1014,30 @@ ndhss_status gmres_batched_run(const FactorData& F, const int32_t* rowptr, const
         ++napply;
         dots(t, 1, t, n2, pact);
         bcycle_kernel<V><<<qb, 256, 0, st>>>(Q, R + 1, n2, g, bs);
-        bscale_kernel<V><<<nseg, 256, 0, st>>>(d_seg, pact, bs, t, Vb);
+        bscale_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, pact, bs, t, Vb);
         NDHSS_LAUNCH_CHECK("bscale_kernel");
         int jend = 0;
         for (int j = 0; j < R; ++j) {
             bpact_kernel<<<pb, 256, 0, st>>>(nsys, bs, pact);
-            spmm_kernel<V><<<nseg, 256, 0, st>>>(d_seg, pact, rowptr, col, vals, Vb + (int64_t)j * nm, w);
+            spmm_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, pact, rowptr, col, vals, Vb + (int64_t)j * nm, w);
             ++nspmv;
             if ((rc = multi_apply_device(F, MR, w, MR, t, MR, mw, st, pact, nprob))) return rc;
             ++napply;
             dots(Vb, j + 1, t, h1, pact);
-            baxpy_kernel<V><<<nseg, 256, 0, st>>>(d_seg, pact, nsys, Vb, nm, j + 1, h1, -1.0, t, nullptr);
+            baxpy_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, pact, nsys, Vb, nm, j + 1, h1, -1.0, t, nullptr);
             dots(Vb, j + 1, t, h2, pact);
-            baxpy_kernel<V><<<nseg, 256, 0, st>>>(d_seg, pact, nsys, Vb, nm, j + 1, h2, -1.0, t, nullptr);
+            baxpy_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, pact, nsys, Vb, nm, j + 1, h2, -1.0, t, nullptr);
             dots(t, 1, t, n2, pact);
             NDHSS_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int), st));
             barnoldi_kernel<V><<<qb, 256, 0, st>>>(Q, j, R, h1, h2, n2, H, g, cs, sn, bs, o.inner * o.tol, o.maxit, cnt);
-            bscale_kernel<V><<<nseg, 256, 0, st>>>(d_seg, pact, bs, t, Vb + (int64_t)(j + 1) * nm);
+            bscale_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, pact, bs, t, Vb + (int64_t)(j + 1) * nm);
             NDHSS_LAUNCH_CHECK("barnoldi_kernel");
             jend = j + 1;
             if ((rc = read_count(&active))) return rc;
             if (active == 0) break;
         }
         bhsolve_kernel<V><<<qb, 256, 0, st>>>(Q, R, H, g, bs, yv);
-        baxpy_kernel<V><<<nseg, 256, 0, st>>>(d_seg, nullptr, nsys, Vb, nm, jend, yv, 1.0, Xi, bs);
+        baxpy_kernel<V><<<seg_grid, 256, 0, st>>>(d_seg, nullptr, nsys, Vb, nm, jend, yv, 1.0, Xi, bs);
         NDHSS_LAUNCH_CHECK("baxpy_kernel");
     }
     bdeinterleave_kernel<V><<<eb, 256, 0, st>>>(n, nrhs, Xi, x, ldx);
@@ -1016,6 +1115,17 @@ ndhss_status build_multi_plan(FactorData& F, cudaStream_t st) {
             }
         }
     F.mj_up_off[2 * (F.depth + 1)] = (int64_t)jobs.size() / 2;
+    // 32-row tiles per level, whatever shape the jobs have (the summation order
+    // depends on it, and must not on the shape)
+    F.mj_up_tiles.assign(F.depth + 1, 0);
+    F.mj_dn_tiles.assign(F.depth + 1, 0);
+    for (int l = 0; l <= F.depth; ++l)
+        for (int s : F.levels[l]) {
+            const int mi = F.m_i(s), mb = F.m_b(s);
+            if (mi == 0) continue;
+            F.mj_up_tiles[l] += ((lowrank(s) ? mi : mi + mb) + 31) / 32;
+            if (mb > 0 && !lowrank(s)) F.mj_dn_tiles[l] += (mi + 31) / 32;
+        }
     for (int l = 0; l <= F.depth; ++l)
         for (int v = 0; v < 2; ++v) {
             F.mj_dn_off[2 * l + v] = (int64_t)jobs.size() / 2;
