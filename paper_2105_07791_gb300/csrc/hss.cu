@@ -1889,7 +1889,21 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
             for (int g = 0; (1 << g) <= RID_MAX_CLUSTER; ++g) nlaunch += grp[g].empty() ? 0 : 1;
             SideFork fork(st, nlaunch > 1 ? nlaunch : 0, F.side_streams);
             HSS_TRY(fork.status);
-            std::vector<std::unique_ptr<DeviceVec<int>>> lists;
+            // the groups' node lists in one table; a level of one group is the level's own list
+            DeviceVec<int> dl(st);
+            std::vector<int> lists;
+            size_t loffs[6] = {};
+            for (int g = 0; g < 5; ++g) {
+                loffs[g] = lists.size();
+                lists.insert(lists.end(), grp[g].begin(), grp[g].end());
+            }
+            loffs[5] = lists.size();
+            lists.insert(lists.end(), big.begin(), big.end());
+            const int* dlist = dflat.p + b;
+            if (nlaunch > 1) {
+                HSS_TRY(dl.upload(lists, st));
+                dlist = dl.p;
+            }
             int li = 0;
             for (int g = 0; (1 << g) <= RID_MAX_CLUSTER; ++g) {
                 if (grp[g].empty()) continue;
@@ -1897,13 +1911,10 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                 cudaStream_t ls = fork.stream(li++);
                 int rcmax = 1;
                 for (int id : grp[g]) rcmax = std::max(rcmax, nodes[id].rows_cap);
-                lists.emplace_back(new DeviceVec<int>(st));
-                DeviceVec<int>& dl = *lists.back();
-                HSS_TRY(dl.upload(grp[g], st));
                 HSS_TRY(fork.start(li - 1));
                 const size_t sm = rid_bytes(rcmax, C);
                 if (C == 1) {
-                    rid_kernel<<<(unsigned)grp[g].size(), Rid<T>::THREADS, sm, ls>>>(dl.p, dnodes.p, ws.p, iws.p, kk.p,
+                    rid_kernel<<<(unsigned)grp[g].size(), Rid<T>::THREADS, sm, ls>>>(dlist + loffs[g], dnodes.p, ws.p, iws.p, kk.p,
                                                                                      rows.p, eps, rank_cap);
                 } else {
                     cudaLaunchConfig_t cfg{};
@@ -1918,7 +1929,7 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                     at[0].val.clusterDim.z = 1;
                     cfg.attrs = at;
                     cfg.numAttrs = 1;
-                    HSS_TRY(cudaLaunchKernelEx(&cfg, rid_kernel, (const int*)dl.p, (const HNode*)dnodes.p,
+                    HSS_TRY(cudaLaunchKernelEx(&cfg, rid_kernel, dlist + loffs[g], (const HNode*)dnodes.p,
                                                ws.p, iws.p, kk.p, (const int*)rows.p, eps, rank_cap));
                 }
                 NDHSS_LAUNCH_CHECK("row_id_cluster_kernel");
@@ -1926,11 +1937,8 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
             }
             if (!big.empty()) {
                 cudaStream_t ls = fork.stream(li++);
-                lists.emplace_back(new DeviceVec<int>(st));
-                DeviceVec<int>& dl = *lists.back();
-                HSS_TRY(dl.upload(big, st));
                 HSS_TRY(fork.start(li - 1));
-                row_id_kernel<T><<<(unsigned)big.size(), 512, smem_base, ls>>>(dl.p, dnodes.p, ws.p, iws.p, kk.p, rows.p,
+                row_id_kernel<T><<<(unsigned)big.size(), 512, smem_base, ls>>>(dlist + loffs[5], dnodes.p, ws.p, iws.p, kk.p, rows.p,
                                                                                 eps, rank_cap, 0);
                 NDHSS_LAUNCH_CHECK("row_id_kernel");
                 HSS_TRY(fork.finish(li - 1));
@@ -1994,18 +2002,24 @@ ndhss_status compress_problems(std::vector<Problem>& probs, bool lowrank, const 
                 yout[i] = static_cast<T*>(fr[i].Zt);
                 lx[i] = ly[i] = fr[i].n;
             }
-            DeviceVec<const T*> dx(st);
-            DeviceVec<T*> dy(st);
-            DeviceVec<int64_t> dlx(st), dly(st);
-            DeviceVec<int> dncs(st);
-            HSS_TRY(dx.upload(xin, st));
-            HSS_TRY(dy.upload(yout, st));
-            HSS_TRY(dlx.upload(lx, st));
-            HSS_TRY(dly.upload(ly, st));
-            HSS_TRY(dncs.upload(ncs, st));
+            // the five per-front arrays in one table
+            std::vector<unsigned char> est(nf * (2 * sizeof(T*) + 2 * sizeof(int64_t) + sizeof(int)));
+            const size_t e_y = nf * sizeof(T*), e_lx = 2 * e_y, e_ly = e_lx + nf * sizeof(int64_t), e_nc = e_ly + nf * sizeof(int64_t);
+            std::memcpy(est.data(), xin.data(), nf * sizeof(T*));
+            std::memcpy(est.data() + e_y, yout.data(), nf * sizeof(T*));
+            std::memcpy(est.data() + e_lx, lx.data(), nf * sizeof(int64_t));
+            std::memcpy(est.data() + e_ly, ly.data(), nf * sizeof(int64_t));
+            std::memcpy(est.data() + e_nc, ncs.data(), nf * sizeof(int));
+            DeviceVec<unsigned char> dest(st);
+            HSS_TRY(dest.upload(est, st));
+            auto* dxp = reinterpret_cast<const T* const*>(dest.p);
+            auto* dyp = reinterpret_cast<T* const*>(dest.p + e_y);
+            auto* dlxp = reinterpret_cast<const int64_t*>(dest.p + e_lx);
+            auto* dlyp = reinterpret_cast<const int64_t*>(dest.p + e_ly);
+            auto* dncp = reinterpret_cast<const int*>(dest.p + e_nc);
             std::vector<char> all(nf, 1);
-            ndhss_status rc = hss_matvec_run<T>(nodes, all, maxlev, dnodes.p, dfr.p, ws.p, ws.p, iws.p, kk.p, rows.p, dx.p,
-                                               dlx.p, dy.p, dly.p, dncs.p, r, (int64_t)kcap, st);
+            ndhss_status rc = hss_matvec_run<T>(nodes, all, maxlev, dnodes.p, dfr.p, ws.p, ws.p, iws.p, kk.p, rows.p, dxp,
+                                               dlxp, dyp, dlyp, dncp, r, (int64_t)kcap, st);
             if (rc != NDHSS_OK) return rc;
         }
         DeviceVec<double> dn(st);
