@@ -32,8 +32,17 @@ namespace ndhss {
 namespace {
 
 constexpr int KMAX = 32;          // restart + 1 <= KMAX
-constexpr int RT = 256;           // reduction block size
-constexpr int RB = 4 * 152;       // reduction grid (four 256-thread blocks per SM)
+// Reductions: one 512-thread block per SM, each on one range of rows (gm_rows).
+// Every block of the Arnoldi kernel adds all blocks' partial sums, so that work
+// grows with the square of the block count, and on a narrow FP64 pipe (an FP64
+// instruction takes a warp 64 clocks) it was much of the step.  Average of the
+// Arnoldi launches of a solve, four 256-thread blocks per SM -> now: 64 x 64
+// real (n = 4k) 15.0 -> 10.3 us, 256 x 256 P1 complex (n = 66k) 25.0 -> 17.9,
+// 256 x 256 P2 complex (n = 263k) 44.6 -> 32.9 (the FP64 pipe's rate from there).
+constexpr int RT = 512;           // reduction block size
+constexpr int RB = 152;           // most blocks of a reduction (one per SM)
+constexpr int GM_ROWS = 128;      // least rows per block: a small system wants few blocks (their barrier, their partials)
+constexpr int GM_MAXD = 16;       // doubles a chunk of basis vectors sums
 constexpr int GM_BARRIER = KMAX / 4 + 1;   // counter word of the Arnoldi kernel's grid barrier
 
 __device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }
@@ -53,6 +62,8 @@ __device__ __forceinline__ c128 warp_sum(c128 v) {
     }
     return v;
 }
+__device__ __forceinline__ double comp(double a, int) { return a; }
+__device__ __forceinline__ double comp(c128 a, int c) { return c ? a.y : a.x; }
 __device__ __forceinline__ double absv(double a) { return fabs(a); }
 __device__ __forceinline__ double absv(c128 a) { return hypot(a.x, a.y); }
 __device__ __forceinline__ c128 cdiv(c128 a, c128 b) { return a * recip(b); }
@@ -248,37 +259,58 @@ __device__ __forceinline__ bool last_block(unsigned* counter, unsigned nblocks) 
     return s_last;
 }
 
-// block sum of one value per thread, valid in thread 0
-template <typename T>
-__device__ __forceinline__ T block_sum(T v) {
-    __shared__ T sred[RT / 32];
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = v;
+// rows of block b of a grid of nb: equal ranges of whole warps
+__device__ __forceinline__ void gm_rows(int n, int64_t& r0, int64_t& r1) {
+    const int64_t per = ((n + (int64_t)gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
+    r0 = min((int64_t)n, per * blockIdx.x);
+    r1 = min((int64_t)n, r0 + per);
+}
+
+// Sums of D values per lane (a power of two, at most 32) over the warp: lane l
+// ends with the sum of value l / (32 / D).  Each of the first log2 D steps
+// halves the values a lane carries (it keeps one half and gets the partner
+// lane's share of it), so the tree issues D - 1 + 5 - log2 D additions instead
+// of 5 D.
+template <int D>
+__device__ __forceinline__ double warp_sums(double (&v)[D]) {
+    const int lane = threadIdx.x & 31;
+    int m = 16;
+#pragma unroll
+    for (int h = D / 2; h >= 1; h >>= 1, m >>= 1) {
+        const bool up = (lane & m) != 0;
+#pragma unroll
+        for (int u = 0; u < h; ++u) {
+            const double send = up ? v[u] : v[u + h];
+            const double keep = up ? v[u + h] : v[u];
+            v[u] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+    }
+#pragma unroll
+    for (; m >= 1; m >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
+    return v[0];
+}
+
+// block sum of one value per thread, valid in thread 0 (`live` false: the
+// whole warp holds zeros)
+__device__ __forceinline__ double block_sum(double v, bool live = true) {
+    __shared__ double sred[RT / 32];
+    if (live) v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = live ? v : 0.0;
     __syncthreads();
-    T s = zero<T>();
-    if (threadIdx.x == 0)
-        for (int q = 0; q < RT / 32; ++q) s += sred[q];
+    double s = 0.0;
+    if (threadIdx.x < 32) {
+        s = threadIdx.x < RT / 32 ? sred[threadIdx.x] : 0.0;
+        s = warp_sum(s);
+    }
     __syncthreads();
     return s;
 }
 
-// sum of the grid's partials by the whole (last) block, four loads in flight
-// per thread, each thread's share in a fixed order, then the block's fixed
-// tree (deterministic); valid in thread 0
-template <typename T>
-__device__ T block_sum_partials(const T* partial, unsigned nb) {
-    T s = zero<T>();
-    unsigned q = threadIdx.x;
-    for (; q + 3 * RT < nb; q += 4 * RT) {
-        const T a0 = ldcg(partial + q), a1 = ldcg(partial + q + RT), a2 = ldcg(partial + q + 2 * RT),
-                a3 = ldcg(partial + q + 3 * RT);
-        s += a0;
-        s += a1;
-        s += a2;
-        s += a3;
-    }
-    for (; q < nb; q += RT) s += ldcg(partial + q);
-    return block_sum(s);
+// sum of the grid's partials (nb <= RB <= RT of them) by the whole (last)
+// block in the block's fixed tree; valid in thread 0
+__device__ __forceinline__ double block_sum_partials(const double* partial, unsigned nb) {
+    static_assert(RB <= RT, "one partial per thread");
+    return block_sum(threadIdx.x < nb ? ldcg(partial + threadIdx.x) : 0.0);
 }
 
 template <typename V>
@@ -362,17 +394,19 @@ __device__ void gm_decide(GmDev<V>* S, double rr, int blk);
 
 // RESTART: r = b - t and the true residual's decisions (gm_decide)
 template <typename V>
-__global__ void __launch_bounds__(RT, 4) gm_resid_kernel(GmDev<V>* S, const V* __restrict__ b, const V* __restrict__ t,
+__global__ void __launch_bounds__(RT, 1) gm_resid_kernel(GmDev<V>* S, const V* __restrict__ b, const V* __restrict__ t,
                                                          V* __restrict__ r, int n, double* __restrict__ partial, int blk) {
     if (S->done || S->bmode != GM_RESTART) return;
     const bool tz = S->spmv_zero != 0;                 // t = A 0 was not formed
     double acc = 0.0;
-    for (int64_t row = (int64_t)blockIdx.x * RT + threadIdx.x; row < n; row += (int64_t)gridDim.x * RT) {
+    int64_t r0, r1;
+    gm_rows(n, r0, r1);
+    for (int64_t row = r0 + threadIdx.x; row < r1; row += RT) {
         const V v = tz ? b[row] : b[row] - t[row];
         r[row] = v;
         acc += norm2(v);
     }
-    const double bs = block_sum(acc);
+    const double bs = block_sum(acc, r0 + (threadIdx.x & ~31u) < r1);
     if (threadIdx.x == 0) partial[blockIdx.x] = bs;
     if (!last_block(S->counter, gridDim.x)) return;
     const double tot = block_sum_partials(partial, gridDim.x);
@@ -432,42 +466,64 @@ __device__ __forceinline__ c128 fmac_conj(c128 v, c128 w, c128 acc) {
 // partial dot products with w over its rows (every block takes the same rows
 // in every pass), one partial per vector and block.  AXPY: w += sum_i
 // raw_i cw[i] with all j + 1 vectors first (the first chunk of the second
-// Gram-Schmidt pass).  Exact-count instantiations: a predicated-off FP64
-// instruction still occupies the FP64 pipe.
+// Gram-Schmidt pass, i0 = 0: its own vectors are loaded once for both).
+// Exact-count instantiations: a predicated-off FP64 instruction still
+// occupies the FP64 pipe.  All values of the chunk are added in one warp tree
+// (warp_sums) and one pass through shared memory; warps without a row skip it.
 template <typename V, int C, bool AXPY>
 __device__ void gm_pass_chunk(V* __restrict__ Vb, int64_t ldv, int n, int j, int i0, const V* cw,
-                              V* __restrict__ partial) {
+                              V* __restrict__ partial, double (*sred)[RT / 32]) {
+    constexpr int NC = sizeof(V) / sizeof(double), D0 = C * NC;
+    constexpr int D = D0 <= 1 ? 1 : D0 <= 2 ? 2 : D0 <= 4 ? 4 : D0 <= 8 ? 8 : 16;
+    static_assert(D0 <= GM_MAXD, "warp_sums of a chunk");
+    constexpr int NW = RT / 32;
+    static_assert(NW == 16, "half a warp adds the warps' sums of a value");
     V* w = Vb + (int64_t)(j + 1) * ldv;
     V acc[C];
 #pragma unroll
     for (int u = 0; u < C; ++u) acc[u] = zero<V>();
-    for (int64_t row = (int64_t)blockIdx.x * RT + threadIdx.x; row < n; row += (int64_t)gridDim.x * RT) {
+    int64_t r0, r1;
+    gm_rows(n, r0, r1);
+    for (int64_t row = r0 + threadIdx.x; row < r1; row += RT) {
         V wv = w[row];
-        if (AXPY) {
-            for (int i = 0; i <= j; ++i) wv = fmac(Vb[row + i * ldv], cw[i], wv);
-            w[row] = wv;
-        }
         V v[C];
 #pragma unroll
         for (int u = 0; u < C; ++u) v[u] = Vb[row + (i0 + u) * ldv];
+        if (AXPY) {
+#pragma unroll
+            for (int u = 0; u < C; ++u) wv = fmac(v[u], cw[u], wv);
+#pragma unroll 4
+            for (int i = C; i <= j; ++i) wv = fmac(Vb[row + i * ldv], cw[i], wv);
+            w[row] = wv;
+        }
 #pragma unroll
         for (int u = 0; u < C; ++u) acc[u] = fmac_conj(v[u], wv, acc[u]);
     }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double d[D];
 #pragma unroll
-    for (int u = 0; u < C; ++u) {
-        const V bs = block_sum(acc[u]);
-        if (threadIdx.x == 0) partial[(int64_t)(i0 + u) * gridDim.x + blockIdx.x] = bs;
+    for (int q = 0; q < D; ++q) d[q] = q < D0 ? comp(acc[q < D0 ? q / NC : 0], q % NC) : 0.0;
+    const bool live = r0 + warp * 32 < r1;               // warp-uniform
+    const double ws = live ? warp_sums<D>(d) : 0.0;
+    __syncthreads();                                     // the previous chunk's sums are read
+    if (lane % (32 / D) == 0) sred[lane / (32 / D)][warp] = ws;
+    __syncthreads();
+    for (int q0 = 2 * warp; q0 < D0; q0 += 2 * NW) {
+        const int q = q0 + (lane >> 4);
+        double v = q < D ? sred[q][lane & 15] : 0.0;
+        for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0 && q < D0)
+            reinterpret_cast<double*>(partial + (int64_t)(i0 + q / NC) * gridDim.x + blockIdx.x)[q % NC] = v;
     }
 }
 
-// basis vectors per chunk: eight real or four complex accumulators and
-// loads in flight keep a thread within the 64 registers of four resident
-// 256-thread blocks per SM
+// basis vectors per chunk: eight real or four complex accumulators and loads
+// in flight (eight complex ones spill at the 128 registers of a 512-thread block)
 template <typename V> constexpr int cgs_width() { return sizeof(V) == 16 ? 4 : 8; }
 
 // one Gram-Schmidt pass's partials: V^H w (AXPY: after w += V cw)
 template <typename V, bool AXPY>
-__device__ void gm_pass(V* Vb, int64_t ldv, int n, int j, const V* cw, V* partial) {
+__device__ void gm_pass(V* Vb, int64_t ldv, int n, int j, const V* cw, V* partial, double (*sred)[RT / 32]) {
     constexpr int CW = cgs_width<V>();
     for (int i0 = 0; i0 <= j; i0 += CW) {
         const bool ax = AXPY && i0 == 0;
@@ -475,8 +531,8 @@ __device__ void gm_pass(V* Vb, int64_t ldv, int n, int j, const V* cw, V* partia
 #define NDHSS_CGS(CC)                                                                               \
     case CC:                                                                                        \
         if constexpr (CC <= CW) {                                                                   \
-            if (ax) gm_pass_chunk<V, CC, true>(Vb, ldv, n, j, i0, cw, partial);                     \
-            else gm_pass_chunk<V, CC, false>(Vb, ldv, n, j, i0, cw, partial);                       \
+            if (ax) gm_pass_chunk<V, CC, true>(Vb, ldv, n, j, i0, cw, partial, sred);                   \
+            else gm_pass_chunk<V, CC, false>(Vb, ldv, n, j, i0, cw, partial, sred);                     \
         }                                                                                           \
         break;
             NDHSS_CGS(1) NDHSS_CGS(2) NDHSS_CGS(3) NDHSS_CGS(4) NDHSS_CGS(5) NDHSS_CGS(6) NDHSS_CGS(7) NDHSS_CGS(8)
@@ -487,7 +543,7 @@ __device__ void gm_pass(V* Vb, int64_t ldv, int n, int j, const V* cw, V* partia
 }
 
 // after a grid barrier: h[i] = scale_i * (sum over blocks of the partials of
-// vector i), i <= j, into shared memory; warp w adds vectors w, w + 8, ...
+// vector i), i <= j, into shared memory; warp w adds vectors w, w + 16, ...
 // (lane-strided in block order, then the warp's fixed tree: every block gets
 // the same values)
 template <typename V>
@@ -495,9 +551,14 @@ __device__ void gm_sum_partials(const V* __restrict__ partial, int j, const doub
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = warp; i <= j; i += RT / 32) {
         V acc = zero<V>();
+#pragma unroll 5
         for (unsigned q = lane; q < gridDim.x; q += 32) acc += ldcg(partial + (int64_t)i * gridDim.x + q);
-        acc = warp_sum(acc);
-        if (lane == 0) h[i] = scale(acc, scl[i]);
+        constexpr int NC = sizeof(V) / sizeof(double);
+        double d[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) d[c] = comp(acc, c);
+        const double hs = warp_sums<NC>(d);
+        if (lane % (32 / NC) == 0) reinterpret_cast<double*>(h + i)[lane / (32 / NC)] = hs * scl[i];
     }
     __syncthreads();
 }
@@ -515,13 +576,16 @@ __device__ void gm_axnorm_step(GmDev<V>* S, V* __restrict__ Vb, int64_t ldv, int
     __syncthreads();
     V* w = Vb + (int64_t)(j + 1) * ldv;
     double acc = 0.0;
-    for (int64_t row = (int64_t)blockIdx.x * RT + threadIdx.x; row < n; row += (int64_t)gridDim.x * RT) {
+    int64_t r0, r1;
+    gm_rows(n, r0, r1);
+    for (int64_t row = r0 + threadIdx.x; row < r1; row += RT) {
         V wv = w[row];
+#pragma unroll 4
         for (int i = 0; i <= j; ++i) wv = fmac(Vb[row + i * ldv], ch[i], wv);
         w[row] = wv;
         acc += norm2(wv);
     }
-    const double bs = block_sum(acc);
+    const double bs = block_sum(acc, r0 + (threadIdx.x & ~31u) < r1);
     if (threadIdx.x == 0) dpartial[blockIdx.x] = bs;
     if (!last_block(S->counter, gridDim.x)) return;
     const double ss = block_sum_partials(dpartial, gridDim.x);
@@ -654,7 +718,7 @@ __device__ bool gm_grid_sync(unsigned* ctr, unsigned target) {
 // host.  All blocks read the solver state's mode words before any block can
 // change them (the last block of each reduction is the only writer).
 template <typename V>
-__global__ void __launch_bounds__(RT, 4) gm_arnoldi_kernel(GmDev<V>* S, V* __restrict__ Vb, int64_t ldv, int n,
+__global__ void __launch_bounds__(RT, 1) gm_arnoldi_kernel(GmDev<V>* S, V* __restrict__ Vb, int64_t ldv, int n,
                                                         V* __restrict__ partial, double* __restrict__ dpartial,
                                                         GmStatus* hstat) {
     const int done = S->done, bmode = S->bmode;
@@ -668,9 +732,11 @@ __global__ void __launch_bounds__(RT, 4) gm_arnoldi_kernel(GmDev<V>* S, V* __res
     }
     if (bmode == GM_RESTART) {
         double acc = 0.0;
-        for (int64_t row = (int64_t)blockIdx.x * RT + threadIdx.x; row < n; row += (int64_t)gridDim.x * RT)
+        int64_t r0, r1;
+        gm_rows(n, r0, r1);
+        for (int64_t row = r0 + threadIdx.x; row < r1; row += RT)
             acc += norm2(Vb[row]);
-        const double bs = block_sum(acc);
+        const double bs = block_sum(acc, r0 + (threadIdx.x & ~31u) < r1);
         if (threadIdx.x == 0) dpartial[blockIdx.x] = bs;
         if (!last_block(S->counter, gridDim.x)) return;
         const double ss = block_sum_partials(dpartial, gridDim.x);
@@ -703,10 +769,11 @@ __global__ void __launch_bounds__(RT, 4) gm_arnoldi_kernel(GmDev<V>* S, V* __res
     const int j = S->j;
     __shared__ double scl[KMAX];
     __shared__ V h1[KMAX], h2[KMAX], cw[KMAX];
+    __shared__ double sred[GM_MAXD][RT / 32];
     if (threadIdx.x <= j) scl[threadIdx.x] = S->scale[threadIdx.x];
     __syncthreads();
     // h1 = V^H w: partials, grid barrier, every block adds them
-    gm_pass<V, false>(Vb, ldv, n, j, nullptr, partial);
+    gm_pass<V, false>(Vb, ldv, n, j, nullptr, partial, sred);
     bool ok = gm_grid_sync(bar, gridDim.x);
     if (ok) {
         gm_sum_partials(partial, j, scl, h1);
@@ -714,7 +781,7 @@ __global__ void __launch_bounds__(RT, 4) gm_arnoldi_kernel(GmDev<V>* S, V* __res
         __syncthreads();
         // w -= V h1, h2 = V^H w (the second pass's partials in their own buffer:
         // other blocks may still be adding the first pass's)
-        gm_pass<V, true>(Vb, ldv, n, j, cw, partial + (int64_t)RB * KMAX);
+        gm_pass<V, true>(Vb, ldv, n, j, cw, partial + (int64_t)RB * KMAX, sred);
         ok = gm_grid_sync(bar, 2 * gridDim.x);
     }
     if (!ok) {
@@ -775,7 +842,7 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
         NDHSS_CUDA_TRY(cudaGetDevice(&dev));
         NDHSS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         NDHSS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gm_arnoldi_kernel<V>, RT, 0));
-        agrid = std::min(RB, per_sm * sms);
+        agrid = std::min({RB, per_sm * sms, (n + GM_ROWS - 1) / GM_ROWS});
         if (agrid < 1) return set_error(NDHSS_ERR_CUDA, "ndhss_gmres: the Arnoldi kernel cannot be resident");
     }
     gm_init_kernel<V><<<1, 1, 0, st>>>(S, R, o.maxit, o.tol, o.inner, o.cycle_rtol);
@@ -811,7 +878,7 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
         gm_spmv_kernel<V><<<sblocks, 256, 0, st>>>(n, rowptr, col, vals, S);
         note_launches(1);
         if (e1) cudaEventRecord(e1, st);
-        gm_resid_kernel<V><<<RB, RT, 0, st>>>(S, b, t, r, n, dpart, blk);
+        gm_resid_kernel<V><<<agrid, RT, 0, st>>>(S, b, t, r, n, dpart, blk);
         note_launches(1);
         if (e2) cudaEventRecord(e2, st);
         rc = apply_device(F, 1, nullptr, n, nullptr, n, awork, st, &S->ind);
