@@ -18,9 +18,10 @@
 // integer below 2^24 for every s, so FP32 accumulation is exact in any order;
 // what is left out (p + q >= 8) is below 2^-60 of the product of the two rows'
 // largest entries per term, under the rounding of a float64 dot product of
-// that length.  The epilogue joins the eight integers into two exact float64
-// values (two FMAs and two additions per element; summing the eight in
-// float64 would make the FP64 pipe the bound again) and adds them to the front.
+// that length.  The epilogue joins the eight integers into two of 51 bits in
+// integer arithmetic, those into one float64 value rounded once (two FMAs,
+// ints_scaled) and adds it to the front: three FP64 instructions per element
+// (summing the eight in float64 would make the FP64 pipe the bound again).
 //
 // Rows with an infinity or a NaN give NaN.
 //
@@ -36,9 +37,12 @@
 // Factorization of the 256 x 256 P2 Helmholtz matrix in complex128: 560 ms with
 // the rank-kb sweep over whole fronts (284 ms of updates), 305 ms with 64-pivot
 // blocks exchanged here, 232 ms with the panels' exchanges as well and the
-// panels over clusters (panel_cluster_kernel); these kernels 41 ms.  A tile takes
-// ~31,000 clocks, about half of it the epilogue's FP64 operations, which do not
-// overlap its MMAs: the accumulators fill the tensor memory.
+// panels over clusters (panel_cluster_kernel).  The epilogue does not overlap a
+// tile's MMAs (the accumulators fill the tensor memory) and was over half of its
+// ~31,000 clocks: front entries loaded eight columns at a time after the MMAs and
+// four FP64 instructions per element.  With the entries loaded while the MMAs run
+// and three instructions, all launches of this kernel in that factorization take
+// 25.7 ms instead of 41.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -197,15 +201,17 @@ tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front
 constexpr uint32_t SW64_HI = (512u >> 4) | 1u << 14 | 4u << 29;
 __device__ __forceinline__ uint32_t sw64_lo(uint32_t saddr) { return (saddr >> 4) | 1u << 16; }
 
-// 2^(f - 1023), and -1.5 2^52 2^(f - 1023)
-__device__ __forceinline__ double pow2_field(int f) { return __longlong_as_double((long long)f << 52); }
-__device__ __forceinline__ double neg_magic_field(int f) {
-    return __longlong_as_double((long long)((1ull << 63) | ((unsigned long long)(f + 52) << 52) | 0x8000000000000ull));
-}
-// the integer x (|x| < 2^51) times 2^(f - 1023), exactly: x + 1.5 2^52 is
-// written down as bits, the FMA takes the constant off again
-__device__ __forceinline__ double int_scaled(long long x, int f) {
-    return fma(__longlong_as_double(x + 0x4338000000000000ll), pow2_field(f), neg_magic_field(f));
+// (hi + lo 2^-32) 2^(f - 1023) for integers |hi|, |lo| < 2^51, rounded once, in
+// two FP64 instructions: x + 1.5 2^52 is written down as bits for both, the
+// first FMA takes both constants off again (hi - 1.5 2^20 is an integer below
+// 2^52: exact)
+__device__ __forceinline__ double ints_scaled(long long hi, long long lo, int f) {
+    const double s = __longlong_as_double((long long)f << 52), s32 = __longlong_as_double((long long)(f - 32) << 52);
+    // -(1.5 2^52 + 1.5 2^20) 2^(f - 1023)
+    const double c = __longlong_as_double(
+        (long long)((1ull << 63) | ((unsigned long long)(f + 52) << 52) | (0x8000000000000ull + 0x180000ull)));
+    const double h = fma(__longlong_as_double(hi + 0x4338000000000000ll), s, c);
+    return fma(__longlong_as_double(lo + 0x4338000000000000ll), s32, h);
 }
 
 template <typename T>
@@ -292,80 +298,79 @@ tc64_gemm_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant
     } else if (warp < 8) {
         // epilogue: warp w takes the tile's rows 32 (w % 4) .. + 31 and columns
         // 32 (w / 4) .. + 31, eight columns of all eight accumulators at a time
+        const int rr = (warp & 3) * 32 + lane, cb = (warp >> 2) * 32;
+        const int64_t grow = m0 + rr;
+        const bool rowok = grow < J.M;
+        const int64_t crow = CPLX ? grow >> 1 : grow;
+        const bool piv = crow >= k0 && crow < k0 + J.w;
+        const int ea = rowok ? rexp[J.ea + crow] : 1;
+        T* out = front + J.out + crow;
+        // the front's entries of this thread (complex: even lanes hold Re, odd
+        // lanes Im of complex row grow / 2; even lanes write the even columns, odd
+        // lanes the odd ones), read while the MMAs run (real: half of them, the
+        // others as these are used; all 32 spill)
+        constexpr int NV = CPLX ? 4 : 8;              // per eight columns
+        constexpr int NO = 16;                        // held at a time
+        T old[NO];
+        auto entry = [&](int q) -> T* {
+            const int64_t col = n0 + cb + (CPLX ? 2 * q + (lane & 1) : q);
+            return rowok && col < J.N ? out + col_of(col, j0, k0, J.w) * J.ldo : nullptr;
+        };
+#pragma unroll
+        for (int q = 0; q < NO; ++q) {
+            const T* ptr = entry(q);
+            old[q] = (ptr && !piv) ? *ptr : zero<T>();
+        }
         const bool ok = tc::bar_wait(&acc_bar, 0);
         tc::fence_after();
         if (!ok || *(volatile int*)&s_abort) {
             if (lane == 0 && atomicCAS(&status->code, 0, (int)NDHSS_ERR_TIMEOUT) == 0) status->node = -1;
         } else {
-            const int rr = (warp & 3) * 32 + lane, cb = (warp >> 2) * 32;
-            const int64_t grow = m0 + rr;
-            const bool rowok = grow < J.M;
-            const int64_t crow = CPLX ? grow >> 1 : grow;
-            const bool piv = crow >= k0 && crow < k0 + J.w;
-            const int ea = rowok ? rexp[J.ea + crow] : 1;
-            T* out = front + J.out;
             const uint32_t t0 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cb;
-            for (int c0 = 0; c0 < 32 && n0 + cb + c0 < J.N; c0 += 8) {
-                long long hi[8], lo[8];
+#pragma unroll
+            for (int c0 = 0; c0 < 32; c0 += 8) {
+                if (n0 + cb + c0 >= J.N) break;
                 uint32_t v[D64][8];
 #pragma unroll
                 for (int g = 0; g < D64; ++g) tc::tmem_ld8_async(t0 + (uint32_t)(g * T64_N + c0), v[g]);
                 tc::tmem_wait_ld();
 #pragma unroll
                 for (int g = 0; g < D64; ++g) tc::tmem_landed(v[g]);
+                double val[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     int d[D64];
 #pragma unroll
                     for (int g = 0; g < D64; ++g) d[g] = __float2int_rn(__uint_as_float(v[g][u]));
                     // |d_0| <= 2^19, |d_1| <= 2^21, |d_2| <= 2^22.6, |d_3| <= 2^23: the pairs fit 32 bits
-                    hi[u] = (long long)(d[0] * 256 + d[1]) * 65536 + (d[2] * 256 + d[3]);
-                    lo[u] = ((long long)d[4] * 256 + d[5]) * 65536 + ((long long)d[6] * 256 + d[7]);
-                }
-                double val[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                    const long long hi = (long long)(d[0] * 256 + d[1]) * 65536 + (d[2] * 256 + d[3]);
+                    const long long lo = ((long long)d[4] * 256 + d[5]) * 65536 + ((long long)d[6] * 256 + d[7]);
                     const int e = ea + s_eb[cb + c0 + u];
                     // V = hi 2^(ea + eb - 36) + lo 2^(ea + eb - 68) with unbiased row
                     // exponents (field - 1022); fields kept inside the normal range
                     // (products of rows below 2^-480 or above 2^480)
                     const int f = min(max(e - 1057, 33), 1990);
-                    val[u] = int_scaled(hi[u], f) + int_scaled(lo[u], f - 32);
+                    val[u] = ints_scaled(hi, lo, f);
                     if (e >= NONFINITE) val[u] = __longlong_as_double(0x7ff8000000000000ll);
                 }
-                if constexpr (CPLX) {
-                    // even lanes hold Re, odd lanes Im of complex row grow / 2; even
-                    // lanes write the even columns, odd lanes the odd ones
-                    const int odd = lane & 1;
-                    T nv[4], old[4];
-                    T* ptr[4];
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) {
+                for (int h = 0; h < NV; ++h) {
+                    T nv;
+                    if constexpr (CPLX) {
+                        const int odd = lane & 1;
                         const double send = odd ? val[2 * h] : val[2 * h + 1];
                         const double recv = __shfl_xor_sync(0xffffffffu, send, 1);
-                        nv[h].x = odd ? recv : val[2 * h];
-                        nv[h].y = odd ? val[2 * h + 1] : recv;
-                        const int64_t col = n0 + cb + c0 + 2 * h + odd;
-                        const int64_t j = col_of(col, j0, k0, J.w);
-                        ptr[h] = (rowok && col < J.N) ? out + j * J.ldo + crow : nullptr;
-                        old[h] = (ptr[h] && !piv) ? *ptr[h] : zero<T>();
+                        nv.x = odd ? recv : val[2 * h];
+                        nv.y = odd ? val[2 * h + 1] : recv;
+                    } else {
+                        nv = val[h];
                     }
-#pragma unroll
-                    for (int h = 0; h < 4; ++h)
-                        if (ptr[h]) *ptr[h] = old[h] + nv[h];
-                } else {
-                    double old[8];
-                    double* ptr[8];
-#pragma unroll
-                    for (int h = 0; h < 8; ++h) {
-                        const int64_t col = n0 + cb + c0 + h;
-                        const int64_t j = col_of(col, j0, k0, J.w);
-                        ptr[h] = (rowok && col < J.N) ? out + j * J.ldo + crow : nullptr;
-                        old[h] = (ptr[h] && !piv) ? *ptr[h] : 0.0;
+                    const int q = c0 / 8 * NV + h;
+                    if (T* ptr = entry(q)) *ptr = old[q % NO] + nv;
+                    if (q + NO < 4 * NV) {
+                        const T* ptr = entry(q + NO);
+                        old[q % NO] = (ptr && !piv) ? *ptr : zero<T>();
                     }
-#pragma unroll
-                    for (int h = 0; h < 8; ++h)
-                        if (ptr[h]) *ptr[h] = old[h] + val[h];
                 }
             }
         }
