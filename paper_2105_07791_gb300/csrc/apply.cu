@@ -126,7 +126,14 @@ constexpr int SUB_MI = 128, SUB_MB = 512;   // largest node
 // P1 Helmholtz, compressed FP32, 151 -> 122 us; 192 x 192 elastic 187 -> 146;
 // 256 x 256 P2 in dense FP64 1209 -> 1005; 1024 roots are slower again).
 // Problems with fewer bottom nodes run per-node tasks all the way down.
-constexpr int SUB_MIN_ROOTS = 512;
+// FP64 problems whose subtrees would get small (under SUB_FP64_DOFS unknowns
+// each) take fewer and larger ones, down to SUB_MIN_ROOTS_FP64: the level tasks
+// that 512 leave over cost more than the unevenness (one apply with 512 / 256 /
+// 128 roots: P2 Helmholtz 87 x 56, n = 20k, 256 / 238 / 230 us; 128 x 128, n =
+// 66k, 398 / 373 / 445; P1 Poisson 250 x 250, n = 62k, 186 / 174 / 181; 120 x
+// 120, n = 14k, 117 / 113 / 113).  FP32 fronts do not gain: 129 x 75 73 / 77 / 77,
+// 87 x 56 95 / 94 / 93, 180 x 180 P2 153 / 169 / 169.
+constexpr int SUB_MIN_ROOTS = 512, SUB_MIN_ROOTS_FP64 = 128, SUB_FP64_DOFS = 300;
 // per-node counters (NCNT arrays of nnodes each) and what signals them
 enum : int { CN_UP = 0, CN_DOT, CN_DIAG, CN_DDOT, CN_FIN, CN_DPART, NCNT };
 constexpr int TK_SHIFT = 25;       // entry word 0 = kind << TK_SHIFT | node (5 bits of kind)
@@ -1473,7 +1480,9 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
                 Ls = l;
             }
             // enough subtrees to fill the GPU (deeper levels have more of them)
-            while (Ls <= F.depth && (int)F.levels[Ls].size() < SUB_MIN_ROOTS) ++Ls;
+            const int min_roots =
+                F.prec == NDHSS_FP64 ? std::clamp(F.n / SUB_FP64_DOFS, SUB_MIN_ROOTS_FP64, SUB_MIN_ROOTS) : SUB_MIN_ROOTS;
+            while (Ls <= F.depth && (int)F.levels[Ls].size() < min_roots) ++Ls;
         }
         if (Ls <= F.depth) {
             // the pivot order of every interior block (final: the factorization
