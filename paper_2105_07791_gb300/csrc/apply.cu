@@ -1354,7 +1354,7 @@ ndhss_status apply_run(const FactorData& F, int32_t nrhs, const V* x, int64_t ld
             (int32_t)F.ulv_recs.size(), F.d_need, reinterpret_cast<int32_t*>(w + WL.ctl), F.d_apply_err};
     const size_t ctl_bytes = sizeof(int32_t) * (CTL_WORDS + (size_t)NCNT * F.nnodes + 2 * F.ulv_recs.size());
     for (int r = 0; r < nrhs; ++r) {
-        NDHSS_CUDA_TRY(cudaMemsetAsync(S.ctl, 0, ctl_bytes, st));
+        if (!ind) NDHSS_CUDA_TRY(cudaMemsetAsync(S.ctl, 0, ctl_bytes, st));
         apply_dataflow_kernel<T, V><<<(unsigned)F.sched_grid, AT, smem, st>>>(C, S, F.n, x + r * ldx, y + r * ldy, wy, wz,
                                                                               tup, tdn, dpart, us, vlen, ind);
         NDHSS_LAUNCH_CHECK("apply_dataflow_kernel");
@@ -1822,6 +1822,12 @@ ndhss_status apply_check_error(const FactorData& F, const char* who) {
 }
 
 size_t apply_work_bytes(const FactorData& F) { return work_layout(F).total; }
+
+void* apply_control(const FactorData& F, void* d_work, int64_t* words16) {
+    const WorkLayout WL = work_layout(F);
+    *words16 = (int64_t)(WL.total - WL.ctl) / 16;
+    return static_cast<unsigned char*>(d_work) + WL.ctl;
+}
 
 ndhss_status apply_device(const FactorData& F, int32_t nrhs, const void* d_x, int64_t ldx, void* d_y, int64_t ldy,
                           void* d_work, cudaStream_t st, const ApplyInd* ind) {

@@ -191,10 +191,9 @@ static ndhss_status conj_inplace(c128* v, int64_t n, cudaStream_t st) {
 // state decides what each block does, so no launch waits for a decision
 // taken on the host:
 //   begin     (RESTART with a finished cycle: x += V y; chooses the vectors
-//             of the SpMV and the apply below)
-//   SpMV      t = s A v  (RESTART: v = x, s = 1; STEP: v = raw basis vector
-//             j, s its scale)
-//   resid     RESTART: r = b - t, ||r||, the float64 true residual decides
+//             of the SpMV and the apply below; zeroes the apply's control words)
+//   SpMV      STEP: t = s A v, v the raw basis vector j, s its scale;
+//             RESTART: r = b - A x, ||r||, the float64 true residual decides
 //             convergence, maxit and the cycle tolerances
 //   apply     RESTART: V_0 = P^{-1} r;  STEP: V_{j+1} = P^{-1} t
 //   dot       RESTART: beta = ||V_0||, g = beta e_1;  STEP: h1 = V^H w
@@ -292,14 +291,15 @@ __device__ __forceinline__ double warp_sums(double (&v)[D]) {
 
 // block sum of one value per thread, valid in thread 0 (`live` false: the
 // whole warp holds zeros)
+template <int NT = RT>
 __device__ __forceinline__ double block_sum(double v, bool live = true) {
-    __shared__ double sred[RT / 32];
+    __shared__ double sred[NT / 32];
     if (live) v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = live ? v : 0.0;
     __syncthreads();
     double s = 0.0;
     if (threadIdx.x < 32) {
-        s = threadIdx.x < RT / 32 ? sred[threadIdx.x] : 0.0;
+        s = threadIdx.x < NT / 32 ? sred[threadIdx.x] : 0.0;
         s = warp_sum(s);
     }
     __syncthreads();
@@ -337,8 +337,10 @@ __global__ void gm_init_kernel(GmDev<V>* S, int R, int maxit, double tol, double
 
 template <typename V>
 __global__ void __launch_bounds__(256) gm_begin_kernel(GmDev<V>* S, V* __restrict__ x, const V* __restrict__ Vb, int64_t ldv,
-                                                       V* t, V* r, int n, int blk) {
+                                                       V* t, V* r, int n, int blk, int4* __restrict__ ctl, int64_t nctl) {
     if (S->done) return;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nctl; q += (int64_t)gridDim.x * blockDim.x)
+        ctl[q] = make_int4(0, 0, 0, 0);
     const int mode = S->mode;
     if (mode == GM_RESTART && S->have_cycle) {
         // x += V y, V_i = scale_i raw_i (y solved when the cycle ended)
@@ -374,44 +376,44 @@ __global__ void __launch_bounds__(256) gm_begin_kernel(GmDev<V>* S, V* __restric
     }
 }
 
-// t = s A v with v, t, s chosen by gm_begin (see spmv_kernel)
-template <typename V>
-__global__ void __launch_bounds__(256) gm_spmv_kernel(int n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                                      const V* __restrict__ vals, const GmDev<V>* S) {
-    if (S->done || S->spmv_zero) return;
-    const V* __restrict__ x = S->spmv_in;
-    V* __restrict__ y = S->spmv_out;
-    const double sc = S->spmv_scale;
-    const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = gt / SP_TPR;
-    const int lane = (int)(gt % SP_TPR);
-    const V acc = spmv_row<V, SP_TPR, SP_U>(row < n, row, lane, rowptr, col, vals, x);
-    if (row < n && lane == 0) y[row] = scale(acc, sc);
-}
-
 template <typename V>
 __device__ void gm_decide(GmDev<V>* S, double rr, int blk);
 
-// RESTART: r = b - t and the true residual's decisions (gm_decide)
+// STEP: t = s A v with v, t, s chosen by gm_begin (see spmv_kernel).  RESTART:
+// r = b - A x (x = 0 before the first cycle: no product) and, in the last block
+// to finish, the true residual's decisions (gm_decide): the row is at hand, and
+// a launch of its own for them, which most blocks of a solve do not need, costs
+// 5 us with its gap.
+constexpr int GM_SPT = 256;
 template <typename V>
-__global__ void __launch_bounds__(RT, 1) gm_resid_kernel(GmDev<V>* S, const V* __restrict__ b, const V* __restrict__ t,
-                                                         V* __restrict__ r, int n, double* __restrict__ partial, int blk) {
-    if (S->done || S->bmode != GM_RESTART) return;
-    const bool tz = S->spmv_zero != 0;                 // t = A 0 was not formed
-    double acc = 0.0;
-    int64_t r0, r1;
-    gm_rows(n, r0, r1);
-    for (int64_t row = r0 + threadIdx.x; row < r1; row += RT) {
-        const V v = tz ? b[row] : b[row] - t[row];
-        r[row] = v;
-        acc += norm2(v);
+__global__ void __launch_bounds__(GM_SPT) gm_spmv_kernel(int n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                                         const V* __restrict__ vals, GmDev<V>* S, const V* __restrict__ b,
+                                                         V* __restrict__ r, double* __restrict__ partial, int blk) {
+    if (S->done) return;
+    const int64_t gt = (int64_t)blockIdx.x * GM_SPT + threadIdx.x;
+    const int64_t row = gt / SP_TPR;
+    const int lane = (int)(gt % SP_TPR);
+    const bool mine = row < n && lane == 0;
+    V acc = zero<V>();
+    if (!S->spmv_zero) acc = spmv_row<V, SP_TPR, SP_U>(row < n, row, lane, rowptr, col, vals, S->spmv_in);
+    if (S->bmode != GM_RESTART) {
+        if (mine) S->spmv_out[row] = scale(acc, S->spmv_scale);
+        return;
     }
-    const double bs = block_sum(acc, r0 + (threadIdx.x & ~31u) < r1);
+    double rr = 0.0;
+    if (mine) {
+        const V v = b[row] - acc;
+        r[row] = v;
+        rr = norm2(v);
+    }
+    const double bs = block_sum<GM_SPT>(rr);
     if (threadIdx.x == 0) partial[blockIdx.x] = bs;
     if (!last_block(S->counter, gridDim.x)) return;
-    const double tot = block_sum_partials(partial, gridDim.x);
+    rr = 0.0;
+    for (unsigned q = threadIdx.x; q < gridDim.x; q += GM_SPT) rr += ldcg(partial + q);
+    rr = block_sum<GM_SPT>(rr);
     // a handful of scalar fields: thread 0 works on the state in place
-    if (threadIdx.x == 0) gm_decide(S, tot, blk);
+    if (threadIdx.x == 0) gm_decide(S, rr, blk);
 }
 
 // RESTART: the float64 true residual ||r||^2 = rr decides convergence,
@@ -787,6 +789,7 @@ __global__ void __launch_bounds__(RT, 1) gm_arnoldi_kernel(GmDev<V>* S, V* __res
     if (!ok) {
         if (threadIdx.x == 0) {
             S->done = 4;
+            S->skip = 1;
             hstat->done = 4;
             __threadfence_system();
         }
@@ -827,14 +830,16 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
     V* t = (V*)carve(sizeof(V) * n);
     V* r = (V*)carve(sizeof(V) * n);
     V* part = (V*)carve(sizeof(V) * 2 * RB * KMAX);   // the two Gram-Schmidt passes' partials
-    double* dpart = (double*)carve(sizeof(double) * RB);
+    const unsigned sblocks = (unsigned)(((int64_t)n * SP_TPR + GM_SPT - 1) / GM_SPT);
+    double* dpart = (double*)carve(sizeof(double) * std::max<size_t>(RB, sblocks));
     GmDev<V>* S = (GmDev<V>*)carve(sizeof(GmDev<V>));
     void* awork = carve(apply_work_bytes(F));
+    int64_t nctl = 0;                                 // the apply's control words, zeroed by gm_begin_kernel
+    void* ctl = apply_control(F, awork, &nctl);
     GmStatus* hst = pinned_status();
     if (!hst) return set_error(NDHSS_ERR_OOM, "ndhss_gmres: pinned status words");
     hst[0] = hst[1] = GmStatus{0, 0, 0, 0};
     const int eb = std::min((n + 255) / 256, 4 * 152);
-    const unsigned sblocks = (unsigned)(((int64_t)n * SP_TPR + 255) / 256);
     // the Arnoldi kernel's grid: every block resident at once (its grid barriers)
     int agrid = 0;
     {
@@ -870,16 +875,14 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
     const int max_blocks = std::min(GM_MAX_BLOCKS, 2 * o.maxit + 4);
     int nblk = 0;
     for (int blk = 0; blk < max_blocks && rc == NDHSS_OK; ++blk) {
-        gm_begin_kernel<V><<<eb, 256, 0, st>>>(S, x, Vb, ldv, t, r, n, blk);
+        gm_begin_kernel<V><<<eb, 256, 0, st>>>(S, x, Vb, ldv, t, r, n, blk, (int4*)ctl, nctl);
         note_launches(1);
         cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr, e3 = nullptr;
         if (o.timing) { e0 = ev(); e1 = ev(); e2 = ev(); e3 = ev(); }
         if (e0) cudaEventRecord(e0, st);
-        gm_spmv_kernel<V><<<sblocks, 256, 0, st>>>(n, rowptr, col, vals, S);
+        gm_spmv_kernel<V><<<sblocks, GM_SPT, 0, st>>>(n, rowptr, col, vals, S, b, r, dpart, blk);
         note_launches(1);
         if (e1) cudaEventRecord(e1, st);
-        gm_resid_kernel<V><<<agrid, RT, 0, st>>>(S, b, t, r, n, dpart, blk);
-        note_launches(1);
         if (e2) cudaEventRecord(e2, st);
         rc = apply_device(F, 1, nullptr, n, nullptr, n, awork, st, &S->ind);
         if (rc != NDHSS_OK) break;
@@ -954,7 +957,7 @@ size_t gmres_work_bytes(const FactorData& F, int R, size_t vsz) {
     add(vsz * F.n);
     add(vsz * F.n);
     add(vsz * 2 * RB * KMAX);
-    add(8 * RB);
+    add(8 * std::max<size_t>(RB, ((size_t)F.n * SP_TPR + GM_SPT - 1) / GM_SPT));
     add(std::max(sizeof(GmDev<double>), sizeof(GmDev<c128>)));
     add(apply_work_bytes(F));
     return b;
