@@ -40,7 +40,14 @@ namespace {
 
 constexpr int KBMAX = 32;
 constexpr int PANEL_THREADS = 512;
-constexpr int PREP_WARPS = 8;
+// panel_prep_kernel is a chain of dependent loads per column (row map, rows, the
+// interchanged rows back, products).  In levels of many fronts a launch has at
+// most PREP_CTAS CTAs (four waves; more only reload the tables) and a warp
+// takes four columns (complex128: two) at once; in fronts above PREP_WIDE rows
+// a whole CTA packs a pivot column.  All launches of a factorization, a warp per
+// column and pivot column always -> now: 512 x 512 P2 Helmholtz (dense, complex64)
+// 7.8 -> 4.7 ms, 256 x 256 P2 complex128 4.5 -> 2.7, complex64 2.0 -> 1.5.
+constexpr int PREP_WARPS = 8, PREP_WIDE = 512, PREP_CTAS = 4 * 8 * 152;
 constexpr int GT = 64;          // gemm tile
 constexpr int MAX_GRID_YZ = 65535;   // largest grid y or z dimension
 constexpr int GK = 16;          // gemm k chunk
@@ -580,7 +587,7 @@ panel_cluster_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict_
     if (rk == 0 && tid == 0) sm[0] = s_na;
 }
 
-template <typename T>
+template <typename T, int PREP_U>
 __global__ void __launch_bounds__(PREP_WARPS * 32)
 panel_prep_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ node,
                   const int64_t* __restrict__ foff, T* __restrict__ front, const int32_t* __restrict__ swapmap,
@@ -600,7 +607,8 @@ panel_prep_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ n
     const int kbp = min(kb, m_i - k0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const T* Ai = ainv_buf + (size_t)li * KBMAX * KBMAX;
-    for (int q = tid; q < KBMAX * KBMAX; q += blockDim.x) s_ai[q] = Ai[q];
+    for (int q = tid; q < kbp * KBMAX; q += blockDim.x)
+        if (q % KBMAX < kbp) s_ai[q] = Ai[q];
     const int32_t* sm = swapmap + (size_t)li * (4 * KBMAX + 1);
     const int na = sm[0];
     for (int a = tid; a < na; a += blockDim.x) {
@@ -611,41 +619,80 @@ panel_prep_kernel(const int32_t* __restrict__ lev, const int32_t* __restrict__ n
     T* F = front + foff[s];
     T* C = cbuf + woff[li] * KBMAX;     // m x kbp, ld m
     T* Z = zbuf + woff[li] * KBMAX;     // kbp x m, ld KBMAX
-    for (int64_t j = (int64_t)blockIdx.x * PREP_WARPS + warp; j < m; j += (int64_t)gridDim.x * PREP_WARPS) {
-        T* Fj = F + j * m;
-        T v0 = zero<T>(), v1 = zero<T>();
-        if (lane < na) v0 = Fj[s_org[lane]];
-        if (lane + 32 < na) v1 = Fj[s_org[lane + 32]];
-        __syncwarp();
-        if (lane < na) Fj[s_rows[lane]] = v0;
-        if (lane + 32 < na) Fj[s_rows[lane + 32]] = v1;
-        __syncwarp();
-        if (j < zlo || j >= zhi) continue;
-        if (j >= k0 && j < k0 + kbp) {
-            const int cidx = (int)(j - k0);
-            // the whole pivot column: eight rows per lane loaded before they are
-            // stored (one load-store pair at a time waits out the latency m / 32 times)
-            for (int64_t i0 = lane; i0 < m; i0 += 32 * 8) {
-                T v[8];
+    // rows i0, i0 + step, ... of pivot column cidx into C, eight loaded before
+    // they are stored
+    auto pack_column = [&](const T* Fj, int cidx, int64_t i0, int64_t step) {
+        for (; i0 < m; i0 += step * 8) {
+            T v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int64_t i = i0 + 32 * u;
-                    v[u] = i < m ? Fj[i] : zero<T>();
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int64_t i = i0 + 32 * u;
-                    if (i >= m) continue;
-                    if (i >= k0 && i < k0 + kbp) v[u] = (i - k0 == cidx) ? one<T>() : zero<T>();
-                    C[(int64_t)cidx * m + i] = v[u];
-                }
+            for (int u = 0; u < 8; ++u) {
+                const int64_t i = i0 + step * u;
+                v[u] = i < m ? Fj[i] : zero<T>();
             }
-            if (lane < kbp) Z[j * KBMAX + lane] = s_ai[cidx * KBMAX + lane];
-        } else {
-            const T w = lane < kbp ? Fj[k0 + lane] : zero<T>();
-            T acc = zero<T>();
-            for (int l = 0; l < kbp; ++l) acc = fmac(s_ai[l * KBMAX + (lane < kbp ? lane : 0)], shfl_idx(w, l), acc);
-            if (lane < kbp) Z[j * KBMAX + lane] = -acc;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int64_t i = i0 + step * u;
+                if (i >= m) continue;
+                if (i >= k0 && i < k0 + kbp) v[u] = (i - k0 == cidx) ? one<T>() : zero<T>();
+                C[(int64_t)cidx * m + i] = v[u];
+            }
+        }
+    };
+    const bool wide = m > PREP_WIDE;
+    if (wide)
+        for (int cidx = blockIdx.x; cidx < kbp; cidx += gridDim.x) {
+            T* Fj = F + (k0 + cidx) * m;
+            if (warp == 0) {
+                T v0 = zero<T>(), v1 = zero<T>();
+                if (lane < na) v0 = Fj[s_org[lane]];
+                if (lane + 32 < na) v1 = Fj[s_org[lane + 32]];
+                __syncwarp();
+                if (lane < na) Fj[s_rows[lane]] = v0;
+                if (lane + 32 < na) Fj[s_rows[lane + 32]] = v1;
+                if (lane < kbp) Z[(k0 + cidx) * (int64_t)KBMAX + lane] = s_ai[cidx * KBMAX + lane];
+            }
+            __syncthreads();
+            pack_column(Fj, cidx, tid, PREP_WARPS * 32);
+        }
+    const int64_t step = (int64_t)gridDim.x * PREP_WARPS;
+    for (int64_t j0 = (int64_t)blockIdx.x * PREP_WARPS + warp; j0 < m; j0 += PREP_U * step) {
+        T v0[PREP_U], v1[PREP_U], w[PREP_U];
+        bool mine[PREP_U], piv[PREP_U], zc[PREP_U];             // warp-uniform
+#pragma unroll
+        for (int u = 0; u < PREP_U; ++u) {
+            const int64_t j = j0 + u * step;
+            piv[u] = j >= k0 && j < k0 + kbp;
+            mine[u] = j < m && !(wide && piv[u]);
+            zc[u] = mine[u] && j >= zlo && j < zhi;
+            const T* Fj = F + j * m;
+            v0[u] = mine[u] && lane < na ? Fj[s_org[lane]] : zero<T>();
+            v1[u] = mine[u] && lane + 32 < na ? Fj[s_org[lane + 32]] : zero<T>();
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < PREP_U; ++u) {
+            T* Fj = F + (j0 + u * step) * m;
+            if (mine[u] && lane < na) Fj[s_rows[lane]] = v0[u];
+            if (mine[u] && lane + 32 < na) Fj[s_rows[lane + 32]] = v1[u];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < PREP_U; ++u)
+            w[u] = zc[u] && !piv[u] && lane < kbp ? F[(j0 + u * step) * m + k0 + lane] : zero<T>();
+#pragma unroll
+        for (int u = 0; u < PREP_U; ++u) {
+            if (!zc[u]) continue;
+            const int64_t j = j0 + u * step;
+            if (piv[u]) {
+                const int cidx = (int)(j - k0);
+                pack_column(F + j * m, cidx, lane, 32);
+                if (lane < kbp) Z[j * KBMAX + lane] = s_ai[cidx * KBMAX + lane];
+            } else {
+                T acc = zero<T>();
+                for (int l = 0; l < kbp; ++l)
+                    acc = fmac(s_ai[l * KBMAX + (lane < kbp ? lane : 0)], shfl_idx(w[u], l), acc);
+                if (lane < kbp) Z[j * KBMAX + lane] = -acc;
+            }
         }
     }
 }
@@ -1124,7 +1171,8 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
         // its pivots), so the FP64 pipe updates the panel's own columns only (256 x
         // 256 P2 Helmholtz, complex128: updates 50 -> 23 ms, exchanges 24 -> 41).
         const bool inner = tcl && F.prec == NDHSS_FP64 && mimax >= TC64_INNER_MIN;
-        const int pgx = (int)std::min<int64_t>((mmax + PREP_WARPS - 1) / PREP_WARPS, 1024);
+        const int pgx = (int)std::min<int64_t>({(mmax + PREP_WARPS - 1) / PREP_WARPS, 1024,
+                                                std::max<int64_t>(1, PREP_CTAS / std::max(1, std::min(L, MAX_GRID_YZ)))});
         for (int64_t k0 = 0; k0 < mimax;) {
             const int64_t s0 = tcl ? k0 / okb * okb : 0;     // the outer block's first pivot
             // panels in registers have a fixed largest width, those in shared memory
@@ -1160,7 +1208,10 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
                 NDHSS_LAUNCH_CHECK("panel kernel");
                 tm.end(2);
                 tm.begin();
-                panel_prep_kernel<T><<<dim3(pgx, Lc), PREP_WARPS * 32, 0, st>>>(levc, F.d_node, F.d_foff, front,
+                // one column per warp where the grid has a warp for each
+                constexpr int PREP_UT = sizeof(T) <= 8 ? 4 : 2;
+                const auto prep = pgx * PREP_WARPS >= mmax ? panel_prep_kernel<T, 1> : panel_prep_kernel<T, PREP_UT>;
+                prep<<<dim3(pgx, Lc), PREP_WARPS * 32, 0, st>>>(levc, F.d_node, F.d_foff, front,
                                                                                d_swapmap, d_ainv, d_cbuf, d_zbuf, woffc,
                                                                                (int)k0, kb, inner ? (int)k0 : (int)s0, inner ? kb : kb2);
                 NDHSS_LAUNCH_CHECK("panel_prep_kernel");

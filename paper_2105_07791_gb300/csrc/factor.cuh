@@ -181,7 +181,7 @@ ndhss_status apply_device(const FactorData& F, int32_t nrhs, const void* d_x, in
                           void* d_y, int64_t ldy, void* d_work, cudaStream_t st, const ApplyInd* ind = nullptr);
 size_t apply_work_bytes(const FactorData& F);
 // The control words within an apply's work area, in 16-byte words: whoever
-// passes `ind` zeroes them on the stream before each apply_device (a solver's
+// passes `ind` (one vector per call) zeroes them on the stream before (a solver's
 // own kernel does it on the way; a memset is a launch and a gap of 4 us).
 void* apply_control(const FactorData& F, void* d_work, int64_t* words16);
 // Builds and uploads the dataflow queue once the factor (and its low-rank
