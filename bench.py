@@ -389,7 +389,7 @@ def run_gpu(a):
         {"kernel": "gm_spmv_kernel (FP64 CSR, complex128; inside the GMRES solves)", "bound": "hbm", "unit": "GB/s",
          "achieved": sp_bytes / (sp_one / 1e3) / 1e9 if sp_one > 0 else None, "peak": pk["hbm_gbs"],
          "peak_kind": f"hbm_gbs, {pk_kind}", "algorithmic": "20 B per entry (value, column) + 36 B per row (row "
-         "pointer, x, y), x read once", "algorithmic_bytes_per_launch": sp_bytes, "avg_launch_ms": sp_one,
+         "pointer, x, y), x read once; a restart's product also forms the residual in that time", "algorithmic_bytes_per_launch": sp_bytes, "avg_launch_ms": sp_one,
          "fp64": {"flops": sp_flops, "achieved_tflops": sp_flops / (sp_one / 1e3) / 1e12 if sp_one > 0 else None,
                   "peak_tflops": fp64_peak, "note": "4 flops per real entry, 8 per complex entry; FP64 FMA rate "
                   "measured in this run"}},

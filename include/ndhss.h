@@ -52,7 +52,10 @@ typedef enum { NDHSS_R64 = 0, NDHSS_C128 = 1 } ndhss_vtype;
 /* Factor storage / arithmetic.  GMRES vectors, the sparse product and the
  * true residual are always float64 (complex128). */
 typedef enum {
-    NDHSS_FP64 = 0,      /* fronts in float64 / complex128, FP64 arithmetic           */
+    NDHSS_FP64 = 0,      /* fronts in float64 / complex128; R, L, S of the larger fronts
+                            as exact integer products on the BF16 tensor cores (62
+                            bits below each row's largest entry: float64-accurate
+                            products), the rest FP64 arithmetic                    */
     NDHSS_FP32 = 1,      /* fronts in float32 / complex64; R, L, S of the larger fronts
                             on the TF32 tensor cores with each operand split in two
                             rounded TF32 parts (hi*hi + hi*lo + lo*hi, FP32
@@ -117,7 +120,8 @@ typedef struct {
     double true_relres;         /* final float64 ||b - A x|| / ||b||                   */
     double precond_relres;      /* last ||P^{-1}(b - A x)|| / ||P^{-1} b|| estimate    */
     int32_t napply, nspmv;      /* preconditioner applies / sparse products issued     */
-    double apply_ms, spmv_ms;   /* their summed device time (only when timing = 1)     */
+    double apply_ms, spmv_ms;   /* their summed device time (only when timing = 1; a
+                                   restart's product includes its residual)         */
 } ndhss_gmres_stats;
 
 typedef struct {
@@ -410,7 +414,7 @@ ndhss_status ndhss_gmres(const ndhss_factorization* f, const int32_t* d_rowptr, 
  * ndhss_apply_multi -- y = P^{-1} x for up to 32 right-hand sides at once
  * (Alg. 3.1 with one pass over the factor for all of them): per level,
  * deepest first, z(I^s) = A_ii^{-1} P^T y(I^s) and y(B^s) -= L P^T y(I^s) for
- * every node of the level as 64-row x 32-column tiles; then per level from
+ * every node of the level, all columns of the call at once; then per level from
  * the roots, z(I^s) += R z(B^s).  Nodes with compressed Gauss transforms
  * (R ~ X R(J,:), L = R^T above the switching level) take the low-rank
  * products t = X^T y(I^s), y(B^s) += R(J,:)^T t on the way up and
