@@ -345,13 +345,19 @@ tc64_gemm_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant
                     // |d_0| <= 2^19, |d_1| <= 2^21, |d_2| <= 2^22.6, |d_3| <= 2^23: the pairs fit 32 bits
                     const long long hi = (long long)(d[0] * 256 + d[1]) * 65536 + (d[2] * 256 + d[3]);
                     const long long lo = ((long long)d[4] * 256 + d[5]) * 65536 + ((long long)d[6] * 256 + d[7]);
-                    const int e = ea + s_eb[cb + c0 + u];
                     // V = hi 2^(ea + eb - 36) + lo 2^(ea + eb - 68) with unbiased row
-                    // exponents (field - 1022); fields kept inside the normal range
-                    // (products of rows below 2^-480 or above 2^480)
+                    // exponents (field - 1022).  ints_scaled wants its powers of two
+                    // inside the normal range; what a product below 2^-954 or above
+                    // 2^1003 lacks (a matrix of entries near 2^-960 or 2^960) is put
+                    // on afterwards, rounded once (a shift beyond 2^+-1022 gives zero
+                    // or infinity either way)
+                    const int e = ea + s_eb[cb + c0 + u];
                     const int f = min(max(e - 1057, 33), 1990);
                     val[u] = ints_scaled(hi, lo, f);
-                    if (e >= NONFINITE) val[u] = __longlong_as_double(0x7ff8000000000000ll);
+                    const int shift = e - 1057 - f;
+                    if (shift != 0)
+                        val[u] *= __longlong_as_double(e >= NONFINITE ? 0x7ff8000000000000ll
+                                                                      : (long long)(1023 + min(max(shift, -1022), 1023)) << 52);
                 }
 #pragma unroll
                 for (int h = 0; h < NV; ++h) {
