@@ -53,9 +53,13 @@ typedef enum { NDHSS_R64 = 0, NDHSS_C128 = 1 } ndhss_vtype;
  * true residual are always float64 (complex128). */
 typedef enum {
     NDHSS_FP64 = 0,      /* fronts in float64 / complex128; R, L, S of the larger fronts
-                            as exact integer products on the BF16 tensor cores (62
-                            bits below each row's largest entry: float64-accurate
-                            products), the rest FP64 arithmetic                    */
+                            as exact integer products on the BF16 tensor cores, the
+                            rest FP64 arithmetic.  An operand row keeps 62 bits below
+                            its largest entry, after the eliminated unknowns' scales
+                            are levelled by powers of two: the error of a product is
+                            below 2^-59 per term of the product of the two rows'
+                            largest entries (unknowns on scales 2^80 apart included),
+                            where float64 has 2^-53 of each term itself           */
     NDHSS_FP32 = 1,      /* fronts in float32 / complex64; R, L, S of the larger fronts
                             on the TF32 tensor cores with each operand split in two
                             rounded TF32 parts (hi*hi + hi*lo + lo*hi, FP32

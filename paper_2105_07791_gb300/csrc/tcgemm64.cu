@@ -8,7 +8,7 @@
 // core takes exactly (the error-free transformation of Ozaki, Ogita, Oishi &
 // Rump, Numer. Algorithms 2012, with a shared exponent per row): with e the
 // exponent of the largest entry of the row (a row of the slab, a column of
-// -M(P, :)),
+// -M(P, :)) once the pivots are levelled,
 //
 //      v = 2^(e - 6) sum_{s < 8} d_s 2^(-8 s),   |d_0| <= 64, |d_s| <= 128,
 //
@@ -16,9 +16,21 @@
 // < 8 are accumulated per s in their own tensor-memory accumulator: 36 MMAs
 // per K step.  A sum of at most T64_KB2 x 2 = 128 such terms per pair is an
 // integer below 2^24 for every s, so FP32 accumulation is exact in any order;
-// what is left out (p + q >= 8) is below 2^-60 of the product of the two rows'
-// largest entries per term, under the rounding of a float64 dot product of
-// that length.  The epilogue joins the eight integers into two of 51 bits in
+// what is left out (p + q >= 8) is below 2^-59 of the product of the two rows'
+// largest entries per term: under the rounding of a float64 dot product of that
+// length where no pivot's products are far below the others'.
+//
+// Levelling sees to that.  Unknowns on different scales (A -> D A E, D and E
+// diagonal) multiply column q of M'(:, P) by 1 / D_q and row q of M(P, :) by D_q:
+// the products keep their size, but a row's largest entry is that of the pivot
+// with the smallest D_q, and the others lose bits.  tc64_level_kernel reads the
+// pivots' scales off the inverse of their own block, M'(P, P), whose rows all
+// combine every pivot: with r_p the exponent of the largest entry of its row p,
+// column q goes up by s_q = min_p (r_p - exponent of (p, q)) powers of two and
+// row q of M down by as many (exact: exponents only).  Errors of one exchange
+// relative to D_i E_j, scales over 2^24 / 2^48 / 2^80: 1e-11 / 6e-5 / 1 without
+// levelling, 1e-16 / 7e-16 / 5e-16 with it, 4e-16 in float64.
+//  The epilogue joins the eight integers into two of 51 bits in
 // integer arithmetic, those into one float64 value rounded once (two FMAs,
 // ints_scaled) and adds it to the front: three FP64 instructions per element
 // (summing the eight in float64 would make the FP64 pipe the bound again).
@@ -94,17 +106,52 @@ template <typename T, int KW>
 constexpr int packed_k() { return (Tr<T>::cplx ? 2 : 1) * KW < T64_BK ? T64_BK : (Tr<T>::cplx ? 2 : 1) * KW; }
 
 // ---------------------------------------------------------------- pack
-// v as an integer: v = X 2^(E - 1084), |X| < 2^62, E >= 1 the largest
-// exponent field of the row (subnormals count as field 1)
-__device__ __forceinline__ int64_t to_fixed(double v, int E) {
+// v 2^lev as an integer X: v 2^lev = X 2^(E - 1084), |X| < 2^62, E the largest
+// levelled exponent of the row (level_exp)
+__device__ __forceinline__ int64_t to_fixed(double v, int lev, int E) {
     const uint64_t b = (uint64_t)__double_as_longlong(v);
     const int f = (int)((b >> 52) & 0x7ff);
     const uint64_t mant = (b & 0xfffffffffffffull) | (f ? 1ull << 52 : 0ull);
-    const int sh = 9 - (E - max(f, 1));
+    const int sh = min(9, 9 - (E - max(f, 1) - lev));       // 9 at most but for zeros
     const uint64_t x = sh >= 0 ? mant << sh : sh > -55 ? (mant + (1ull << (-sh - 1))) >> -sh : 0ull;
     return (b >> 63) ? -(int64_t)x : (int64_t)x;
 }
-__device__ __forceinline__ int exp_field(double v) { return (int)((__double2hiint(v) >> 20) & 0x7ff); }
+// exponent field of v 2^lev, subnormals counting as field 1; INT_MIN for zero,
+// NONFINITE for an infinity or a NaN
+__device__ __forceinline__ int level_exp(double v, int lev) {
+    const int f = (int)((__double2hiint(v) >> 20) & 0x7ff);
+    return v == 0.0 ? INT_MIN : f == 0x7ff ? NONFINITE : max(f, 1) + lev;
+}
+__device__ __forceinline__ int level_exp(c128 v, int lev) { return max(level_exp(v.x, lev), level_exp(v.y, lev)); }
+
+// The powers of two s_q that level the pivots of an exchange (top of the file),
+// one CTA per front, KW per front in lev: a few KB to read, bound by latency.
+template <typename T, int KW>
+__global__ void __launch_bounds__(256)
+tc64_level_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front, int k0, int32_t* __restrict__ lev) {
+    __shared__ int ex[KW][KW + 1];
+    __shared__ int rmax[KW];
+    const Front64 P = fronts[blockIdx.x];
+    const int w = P.w;
+    const T* D = front + P.foff + (int64_t)k0 * P.m + k0;
+    for (int q = threadIdx.x; q < w * w; q += 256) ex[q % w][q / w] = level_exp(D[(int64_t)(q / w) * P.m + q % w], 0);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int p = warp; p < w; p += 8) {
+        int r = INT_MIN;
+        for (int q = lane; q < w; q += 32) r = max(r, ex[p][q]);
+        r = __reduce_max_sync(0xffffffffu, r);
+        if (lane == 0) rmax[p] = r;
+    }
+    __syncthreads();
+    for (int q = warp; q < w; q += 8) {
+        int s = INT_MAX;
+        for (int p = lane; p < w; p += 32)
+            if (ex[p][q] != INT_MIN) s = min(s, rmax[p] - ex[p][q]);
+        s = __reduce_min_sync(0xffffffffu, s);
+        if (lane == 0) lev[(int64_t)blockIdx.x * KW + q] = s == INT_MAX ? 0 : min(s, 4096);
+    }
+}
 
 // the low digit of x (-128 .. 127) split off
 __device__ __forceinline__ float next_digit(int64_t& x, bool last) {
@@ -119,8 +166,8 @@ __device__ __forceinline__ float next_digit(int64_t& x, bool last) {
 // the pivots; pivots from w on are zeros.
 template <typename T, int KW>
 __global__ void __launch_bounds__(256)
-tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front, int k0, int j0,
-                 __nv_bfloat16* __restrict__ packed, int32_t* __restrict__ rexp) {
+tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front, const int32_t* __restrict__ lev, int k0,
+                 int j0, __nv_bfloat16* __restrict__ packed, int32_t* __restrict__ rexp) {
     constexpr bool CPLX = Tr<T>::cplx;
     constexpr int CX = CPLX ? 2 : 1;
     constexpr int Kp = packed_k<T, KW>(), KL = Kp / CX;      // packed values and entries of a row
@@ -151,25 +198,32 @@ tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front
     const int64_t a_rows = (int64_t)CX * m;
     const unsigned mask = RW == 1 ? 0xffffffffu : 0xffffu << (16 * sub);
     static_assert(RW == 1 || LPR == 16, "whole or half warps");
+    int lv[UL];
+#pragma unroll
+    for (int u = 0; u < UL; ++u) {
+        const int l = ll + LPR * u;
+        const int s = l < w ? lev[(int64_t)blockIdx.y * KW + l] : 0;
+        lv[u] = is_a ? s : -s;
+    }
     for (int rr = RW * warp + sub; rr < 32; rr += 8 * RW) {
         const int r = r0 + rr;
         T v[UL];
-        int E = 1;
+        int E = INT_MIN;
 #pragma unroll
         for (int u = 0; u < UL; ++u) {
             v[u] = ts[rr][ll + LPR * u];
-            if constexpr (CPLX) E = max(E, max(exp_field(v[u].x), exp_field(v[u].y)));
-            else E = max(E, exp_field(v[u]));
+            E = max(E, level_exp(v[u], lv[u]));
         }
         E = __reduce_max_sync(mask, E);
         if (r >= rows) continue;
-        const bool bad = E == 0x7ff;
+        if (E == INT_MIN) E = 1023;                    // a row of zeros
+        const bool bad = E == NONFINITE;
         if (ll == 0) rexp[P.e0 + (is_a ? 0 : m) + r] = bad ? NONFINITE : E;
 #pragma unroll
         for (int u = 0; u < UL; ++u) {
             const int l = ll + LPR * u;
             if constexpr (CPLX) {
-                int64_t xr = bad ? 0 : to_fixed(v[u].x, E), xi = bad ? 0 : to_fixed(v[u].y, E);
+                int64_t xr = bad ? 0 : to_fixed(v[u].x, lv[u], E), xi = bad ? 0 : to_fixed(v[u].y, lv[u], E);
                 __nv_bfloat162* o0 = reinterpret_cast<__nv_bfloat162*>(
                     packed + (is_a ? P.row0 + 2 * (int64_t)r : P.row0 + D64 * a_rows + r) * Kp + 2 * l);
                 const int64_t ps = (is_a ? a_rows : nb) * (int64_t)(Kp / 2);
@@ -184,7 +238,7 @@ tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front
                     }
                 }
             } else {
-                int64_t x = bad ? 0 : to_fixed(v[u], E);
+                int64_t x = bad ? 0 : to_fixed(v[u], lv[u], E);
                 __nv_bfloat16* o0 = packed + (is_a ? P.row0 + r : P.row0 + D64 * a_rows + r) * Kp + l;
                 const int64_t ps = (is_a ? a_rows : nb) * (int64_t)Kp;
 #pragma unroll
@@ -430,9 +484,10 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
             rt_max = std::max(rt_max, (m + 31) / 32 + (nb + 31) / 32);
         }
         if (fr.empty()) break;
-        // one pool allocation: packed digits, row exponents, then the tables
+        // one pool allocation: packed digits, row exponents and the pivots'
+        // levels, then the tables
         auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
-        const size_t packed_bytes = r256((size_t)rows * Kp * 2), exp_bytes = r256((size_t)nexp * 4);
+        const size_t packed_bytes = r256((size_t)rows * Kp * 2), exp_bytes = r256(((size_t)nexp + fr.size() * KW) * 4);
         const size_t fr_bytes = r256(fr.size() * sizeof(Front64)), job_bytes = r256(jobs.size() * sizeof(Job64));
         const size_t t_bytes = r256(tiles.size() * sizeof(int2));
         std::vector<unsigned char> tab(fr_bytes + job_bytes + t_bytes);
@@ -446,6 +501,7 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
             return set_error(NDHSS_ERR_OOM, "ndhss_factor: %zu bytes of packed tensor-core operands", packed_bytes);
         }
         int32_t* d_exp = reinterpret_cast<int32_t*>(buf + packed_bytes);
+        int32_t* d_lev = d_exp + nexp;
         unsigned char* d_tab = buf + packed_bytes + exp_bytes;
         ndhss_status rc = NDHSS_OK;
         if (cudaMemcpyAsync(d_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -464,8 +520,15 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
                                   CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (rc == NDHSS_OK) {
+            tc64_level_kernel<T, KW><<<(unsigned)fr.size(), 256, 0, st>>>(reinterpret_cast<const Front64*>(d_tab),
+                                                                          static_cast<const T*>(F.d_front), k0, d_lev);
+            const cudaError_t e = cudaGetLastError();
+            note_launches(1);
+            if (e != cudaSuccess) rc = set_error(NDHSS_ERR_CUDA, "launch of tc64_level_kernel failed: %s", cudaGetErrorString(e));
+        }
+        if (rc == NDHSS_OK) {
             tc64_pack_kernel<T, KW><<<dim3((unsigned)rt_max, (unsigned)fr.size()), 256, 0, st>>>(
-                reinterpret_cast<const Front64*>(d_tab), static_cast<const T*>(F.d_front), k0, j0,
+                reinterpret_cast<const Front64*>(d_tab), static_cast<const T*>(F.d_front), d_lev, k0, j0,
                 reinterpret_cast<__nv_bfloat16*>(buf), d_exp);
             const cudaError_t e = cudaGetLastError();
             note_launches(1);
@@ -481,7 +544,7 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
         }
         cudaFreeAsync(buf, st);
         if (rc != NDHSS_OK) return rc;
-        F.launches += 2;
+        F.launches += 3;
         for (const auto& f : fr) F.tc_flops += (Tr<T>::cplx ? 8.0 : 2.0) * (double)f.m * (double)f.nb * f.w;
     }
     return NDHSS_OK;
