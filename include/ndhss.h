@@ -259,6 +259,10 @@ void ndhss_tree_destroy(ndhss_tree* t);
  *              elimination; both are joined back to `stream` and ended
  *              before the call returns)
  *   out        receives a new factor handle holding device memory
+ * Work space from the library's pool beside the factor's own memory: per level
+ * two m x 32 panels of every front; FP64 fronts up to 1 GB of packed operands
+ * (less where there is less: smaller batches of fronts, and a front that finds
+ * no memory by itself is exchanged in float64 without them).
  * Errors: SINGULAR (node reported), OOM, CUDA, INVALID_ARG.
  */
 ndhss_status ndhss_factor(const ndhss_tree* t, int32_t vtype, const int32_t* d_rowptr,

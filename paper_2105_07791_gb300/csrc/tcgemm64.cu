@@ -60,6 +60,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cstdlib>
 #include <vector>
 
 #include "driver.h"
@@ -445,22 +446,74 @@ tc64_gemm_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant
     if (warp == 0) tc::tmem_dealloc(tmem, T64_TMEM_COLS);
 }
 
+// ---------------------------------------------------------------- without packed operands
+// The exchange in float64 on the CUDA cores, straight from the front: a CTA
+// takes the columns [16 blockIdx.x, + 16) of front blockIdx.y, holds -M(P, :) of
+// them in shared memory (no other CTA reads or writes these columns) and walks
+// over the rows, a row per thread.  Taken when there is no memory for packed
+// operands; bound by the FP64 pipe (2 DFMA per clock and SM).
+constexpr int T64_PC = 16;
+template <typename T>
+__global__ void __launch_bounds__(256)
+tc64_plain_kernel(const Front64* __restrict__ fronts, T* __restrict__ front, int k0, int j0) {
+    __shared__ T bs[TC64_KB2][T64_PC];
+    const Front64 P = fronts[blockIdx.y];
+    const int m = P.m, w = P.w, c0 = (int)blockIdx.x * T64_PC;
+    if (c0 >= P.nb) return;
+    T* F = front + P.foff;
+    for (int q = threadIdx.x; q < w * T64_PC; q += 256) {
+        const int l = q % w, c = q / w;
+        bs[l][c] = c0 + c < P.nb ? -F[col_of(c0 + c, j0, k0, w) * m + k0 + l] : zero<T>();
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < m; i += 256) {
+        T acc[T64_PC];
+#pragma unroll
+        for (int c = 0; c < T64_PC; ++c) acc[c] = zero<T>();
+        for (int l = 0; l < w; ++l) {
+            const T a = F[(int64_t)(k0 + l) * m + i];
+#pragma unroll
+            for (int c = 0; c < T64_PC; ++c) acc[c] = fmac(a, bs[l][c], acc[c]);
+        }
+        const bool piv = i >= k0 && i < k0 + w;
+#pragma unroll
+        for (int c = 0; c < T64_PC; ++c) {
+            if (c0 + c >= P.nb) break;
+            T* ptr = F + col_of(c0 + c, j0, k0, w) * m + i;
+            *ptr = piv ? acc[c] : *ptr + acc[c];
+        }
+    }
+}
+
+// Packed operands of one batch of fronts, and no more: they come on top of the
+// factor itself (6 KB per row of a complex128 front and 64 pivots, more than the
+// front's own 16 m bytes up to m = 384), and a batch of this size already has
+// thousands of tiles.  NDHSS_TC64_SCRATCH sets another limit in bytes (0: no
+// packed operands at all).
+int64_t scratch_limit() {
+    const char* e = std::getenv("NDHSS_TC64_SCRATCH");
+    return e ? std::max<int64_t>(0, std::atoll(e)) : (int64_t)1 << 30;
+}
+
 template <typename T, int KW>
 ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0, int width, int j0, int j1,
                             DevStatus* d_status, cudaStream_t st) {
     constexpr int CX = Tr<T>::cplx ? 2 : 1;
     constexpr int64_t Kp = packed_k<T, KW>();
     NDHSS_CUDA_TRY(cudaFuncSetAttribute(tc64_gemm_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T64_SMEM));
-    // fronts in batches whose packed operands stay below 8 GB and the tensor
-    // map's 2^31 rows
-    constexpr int64_t MAX_ROWS = std::min<int64_t>(((int64_t)1 << 31) - 4096, ((int64_t)8 << 30) / (Kp * 2));
+    // fronts in batches whose packed operands stay below the limit and the tensor
+    // map's 2^31 rows; a batch that finds no memory is halved, and a front that
+    // finds none by itself goes without
+    int64_t max_rows = std::min<int64_t>(((int64_t)1 << 31) - 4096, scratch_limit() / (Kp * 2));
     size_t at = 0;
     while (at < nodes.size()) {
         std::vector<Front64> fr;
         std::vector<Job64> jobs;
         std::vector<int2> tiles;
-        int64_t rows = 0, nexp = 0;
-        int rt_max = 0;
+        int64_t rows = 0, nexp = 0, need_max = 0;
+        int rt_max = 0, nb_max = 0;
+        const size_t first = at;
+        bool packed = true;
         for (; at < nodes.size(); ++at) {
             const int s = nodes[at];
             const int mi = F.m_i(s), m = mi + F.m_b(s);
@@ -468,14 +521,15 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
             const int w = std::min(width, mi - k0), nb = std::min(j1 == INT_MAX ? m : mi, j1) - j0 - w;
             if (nb <= 0) continue;                         // the pivots are all of the columns
             const int64_t a_rows = (int64_t)CX * m, need = D64 * (a_rows + nb);
-            if (!fr.empty() && (rows + need > MAX_ROWS || fr.size() >= 65535)) break;
-            if (rows + need >= ((int64_t)1 << 31) - 4096)
-                return set_error(NDHSS_ERR_INVALID_ARG, "ndhss_factor: %lld packed operand rows exceed the tensor map's range",
-                                 (long long)need);
+            if (!fr.empty() && (fr.size() >= 65535 || packed != (need <= max_rows) || (packed && rows + need > max_rows))) break;
+            packed = need <= max_rows;
             fr.push_back({F.foff[s], rows, m, w, nb, (int32_t)nexp});
+            nb_max = std::max(nb_max, nb);
+            if (!packed) continue;
             const Job64 j{(int32_t)rows, (int32_t)a_rows, (int32_t)(rows + D64 * a_rows), nb, (int32_t)a_rows, nb, CX * w,
                           w, F.foff[s], m, (int32_t)nexp, (int32_t)(nexp + m), 0};
             rows += need;
+            need_max = std::max(need_max, need);
             nexp += m + nb;
             const int id = (int)jobs.size();
             jobs.push_back(j);
@@ -487,7 +541,7 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
         // one pool allocation: packed digits, row exponents and the pivots'
         // levels, then the tables
         auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
-        const size_t packed_bytes = r256((size_t)rows * Kp * 2), exp_bytes = r256(((size_t)nexp + fr.size() * KW) * 4);
+        const size_t packed_bytes = r256((size_t)rows * Kp * 2), exp_bytes = packed ? r256(((size_t)nexp + fr.size() * KW) * 4) : 0;
         const size_t fr_bytes = r256(fr.size() * sizeof(Front64)), job_bytes = r256(jobs.size() * sizeof(Job64));
         const size_t t_bytes = r256(tiles.size() * sizeof(int2));
         std::vector<unsigned char> tab(fr_bytes + job_bytes + t_bytes);
@@ -498,14 +552,36 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
         unsigned char* buf = nullptr;
         if (pool_malloc_async((void**)&buf, packed_bytes + exp_bytes + tab.size(), st) != cudaSuccess) {
             cudaGetLastError();
-            return set_error(NDHSS_ERR_OOM, "ndhss_factor: %zu bytes of packed tensor-core operands", packed_bytes);
+            if (!packed) return set_error(NDHSS_ERR_OOM, "ndhss_factor: %zu bytes of front tables", tab.size());
+            max_rows = fr.size() > 1 ? std::max(rows / 2, need_max) : rows - 1;
+            at = first;
+            continue;
         }
         int32_t* d_exp = reinterpret_cast<int32_t*>(buf + packed_bytes);
         int32_t* d_lev = d_exp + nexp;
         unsigned char* d_tab = buf + packed_bytes + exp_bytes;
+        const Front64* d_fr = reinterpret_cast<const Front64*>(d_tab);
+        T* front = static_cast<T*>(F.d_front);
         ndhss_status rc = NDHSS_OK;
         if (cudaMemcpyAsync(d_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
             rc = set_error(NDHSS_ERR_CUDA, "ndhss_factor: upload of the tensor-core tables failed");
+        auto launched = [&](const char* name) {
+            const cudaError_t e = cudaGetLastError();
+            note_launches(1);
+            ++F.launches;
+            if (e != cudaSuccess) rc = set_error(NDHSS_ERR_CUDA, "launch of %s failed: %s", name, cudaGetErrorString(e));
+        };
+        if (!packed) {
+            if (rc == NDHSS_OK) {
+                tc64_plain_kernel<T><<<dim3((unsigned)((nb_max + T64_PC - 1) / T64_PC), (unsigned)fr.size()), 256, 0, st>>>(
+                    d_fr, front, k0, j0);
+                launched("tc64_plain_kernel");
+            }
+            cudaFreeAsync(buf, st);
+            if (rc != NDHSS_OK) return rc;
+            for (const auto& f : fr) F.update_flops += (Tr<T>::cplx ? 8.0 : 2.0) * (double)f.m * (double)f.nb * f.w;
+            continue;
+        }
         CUtensorMap amap, bmap;
         const cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)rows};
         const cuuint64_t strides[1] = {(cuuint64_t)Kp * 2};
@@ -520,31 +596,22 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
                                   CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (rc == NDHSS_OK) {
-            tc64_level_kernel<T, KW><<<(unsigned)fr.size(), 256, 0, st>>>(reinterpret_cast<const Front64*>(d_tab),
-                                                                          static_cast<const T*>(F.d_front), k0, d_lev);
-            const cudaError_t e = cudaGetLastError();
-            note_launches(1);
-            if (e != cudaSuccess) rc = set_error(NDHSS_ERR_CUDA, "launch of tc64_level_kernel failed: %s", cudaGetErrorString(e));
+            tc64_level_kernel<T, KW><<<(unsigned)fr.size(), 256, 0, st>>>(d_fr, front, k0, d_lev);
+            launched("tc64_level_kernel");
         }
         if (rc == NDHSS_OK) {
             tc64_pack_kernel<T, KW><<<dim3((unsigned)rt_max, (unsigned)fr.size()), 256, 0, st>>>(
-                reinterpret_cast<const Front64*>(d_tab), static_cast<const T*>(F.d_front), d_lev, k0, j0,
-                reinterpret_cast<__nv_bfloat16*>(buf), d_exp);
-            const cudaError_t e = cudaGetLastError();
-            note_launches(1);
-            if (e != cudaSuccess) rc = set_error(NDHSS_ERR_CUDA, "launch of tc64_pack_kernel failed: %s", cudaGetErrorString(e));
+                d_fr, front, d_lev, k0, j0, reinterpret_cast<__nv_bfloat16*>(buf), d_exp);
+            launched("tc64_pack_kernel");
         }
         if (rc == NDHSS_OK) {
             tc64_gemm_kernel<T><<<(unsigned)tiles.size(), T64_THREADS, T64_SMEM, st>>>(
                 amap, bmap, reinterpret_cast<const Job64*>(d_tab + fr_bytes),
-                reinterpret_cast<const int2*>(d_tab + fr_bytes + job_bytes), d_exp, k0, j0, static_cast<T*>(F.d_front), d_status);
-            const cudaError_t e = cudaGetLastError();
-            note_launches(1);
-            if (e != cudaSuccess) rc = set_error(NDHSS_ERR_CUDA, "launch of tc64_gemm_kernel failed: %s", cudaGetErrorString(e));
+                reinterpret_cast<const int2*>(d_tab + fr_bytes + job_bytes), d_exp, k0, j0, front, d_status);
+            launched("tc64_gemm_kernel");
         }
         cudaFreeAsync(buf, st);
         if (rc != NDHSS_OK) return rc;
-        F.launches += 3;
         for (const auto& f : fr) F.tc_flops += (Tr<T>::cplx ? 8.0 : 2.0) * (double)f.m * (double)f.nb * f.w;
     }
     return NDHSS_OK;
@@ -554,12 +621,16 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
 
 ndhss_status tc64_block_exchange(FactorData& F, const std::vector<int>& nodes, int k0, int width, int j0, int j1,
                                  DevStatus* d_status, cudaStream_t st) {
-    const bool narrow = width <= TC64_KB1;
-    if (F.vtype == NDHSS_C128)
-        return narrow ? tc64_block_run<c128, TC64_KB1>(F, nodes, k0, width, j0, j1, d_status, st)
-                      : tc64_block_run<c128, TC64_KB2>(F, nodes, k0, width, j0, j1, d_status, st);
-    return narrow ? tc64_block_run<double, TC64_KB1>(F, nodes, k0, width, j0, j1, d_status, st)
-                  : tc64_block_run<double, TC64_KB2>(F, nodes, k0, width, j0, j1, d_status, st);
+    // the packed width by the call's widest pivot block
+    int wmax = 0;
+    for (int s : nodes) wmax = std::max(wmax, std::min(width, F.m_i(s) - k0));
+    auto run = [&](auto v) {
+        using T = decltype(v);
+        return wmax <= TC64_KB1 ? tc64_block_run<T, TC64_KB1>(F, nodes, k0, width, j0, j1, d_status, st)
+               : wmax <= 32     ? tc64_block_run<T, 32>(F, nodes, k0, width, j0, j1, d_status, st)
+                                : tc64_block_run<T, TC64_KB2>(F, nodes, k0, width, j0, j1, d_status, st);
+    };
+    return F.vtype == NDHSS_C128 ? run(c128{}) : run(double{});
 }
 
 }  // namespace ndhss
