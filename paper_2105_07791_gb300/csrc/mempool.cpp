@@ -9,9 +9,10 @@
 // Page-locked staging buffers for small host tables: a copy from pageable
 // memory costs the host several microseconds each, and the compression's
 // rounds upload a dozen tables per round.  A buffer belongs to one call at a
-// time; it is handed out again once the copies of the call before have run
-// (an event on that call's stream).  At most PINNED_KEEP free buffers per
-// process are kept.
+// time and is handed out again once the copies of the call before have run (an
+// event on that call's stream): a call takes an idle one, or a new one while
+// the device has fewer than PINNED_MAX, or does without.  It never waits: the
+// event may lie behind other work of another thread's stream.
 #include <cstdint>
 #include <mutex>
 #include <new>
@@ -60,8 +61,9 @@ cudaError_t pool_malloc_async(void** p, size_t bytes, cudaStream_t st) {
 }
 
 namespace {
-constexpr size_t PINNED_KEEP = 4;
+constexpr int PINNED_MAX = 4;                    // buffers per device, in use or not
 std::mutex g_pinned_mu;
+int g_pinned_count[MAX_DEVICES] = {};
 std::vector<PinnedBuf*>& pinned_free() {
     static std::vector<PinnedBuf*>* v = new std::vector<PinnedBuf*>();     // lives until the process exits
     return *v;
@@ -69,31 +71,37 @@ std::vector<PinnedBuf*>& pinned_free() {
 void pinned_destroy(PinnedBuf* b) {
     if (b->p) cudaFreeHost(b->p);
     if (b->ev) cudaEventDestroy(b->ev);
+    std::lock_guard<std::mutex> lock(g_pinned_mu);
+    --g_pinned_count[b->dev];
     delete b;
 }
 }  // namespace
 
 PinnedBuf* pinned_acquire() {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-    PinnedBuf* b = nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return nullptr;
     {
         std::lock_guard<std::mutex> lock(g_pinned_mu);
         std::vector<PinnedBuf*>& v = pinned_free();
-        for (size_t i = v.size(); i-- > 0 && !b;)
-            if (v[i]->dev == dev) {
-                b = v[i];
-                v.erase(v.begin() + (std::ptrdiff_t)i);
+        for (size_t i = v.size(); i-- > 0;) {
+            if (v[i]->dev != dev) continue;
+            if (cudaEventQuery(v[i]->ev) != cudaSuccess) {
+                cudaGetLastError();              // not ready
+                continue;
             }
+            PinnedBuf* b = v[i];
+            v.erase(v.begin() + (std::ptrdiff_t)i);
+            return b;
+        }
+        if (g_pinned_count[dev] >= PINNED_MAX) return nullptr;
+        ++g_pinned_count[dev];
     }
-    if (b) {
-        if (cudaEventSynchronize(b->ev) == cudaSuccess) return b;
-        cudaGetLastError();
-        pinned_destroy(b);
+    PinnedBuf* b = new (std::nothrow) PinnedBuf();
+    if (!b) {
+        std::lock_guard<std::mutex> lock(g_pinned_mu);
+        --g_pinned_count[dev];
         return nullptr;
     }
-    b = new (std::nothrow) PinnedBuf();
-    if (!b) return nullptr;
     b->dev = dev;
     if (cudaHostAlloc(reinterpret_cast<void**>(&b->p), PINNED_BYTES, cudaHostAllocDefault) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess) {
@@ -106,17 +114,14 @@ PinnedBuf* pinned_acquire() {
 
 void pinned_release(PinnedBuf* b, cudaStream_t st) {
     if (!b) return;
-    bool keep = cudaEventRecord(b->ev, st) == cudaSuccess;
-    if (keep) {
+    if (cudaEventRecord(b->ev, st) == cudaSuccess) {
         std::lock_guard<std::mutex> lock(g_pinned_mu);
-        keep = pinned_free().size() < PINNED_KEEP;
-        if (keep) pinned_free().push_back(b);
+        pinned_free().push_back(b);
+        return;
     }
-    if (!keep) {
-        cudaStreamSynchronize(st);
-        cudaGetLastError();
-        pinned_destroy(b);
-    }
+    cudaStreamSynchronize(st);
+    cudaGetLastError();
+    pinned_destroy(b);
 }
 
 }  // namespace ndhss
