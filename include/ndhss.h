@@ -82,7 +82,8 @@ typedef struct {
     int32_t k0;                 /* initial rank guess of Alg. A.1, e.g. 32             */
     int32_t r;                  /* rank step / estimator samples of Alg. A.1, e.g. 16  */
     int32_t rank_cap;           /* largest HSS rank allowed, e.g. 512                  */
-    int32_t panel;              /* pivot block width of the front kernels, 0 = auto    */
+    int32_t panel;              /* largest pivot block width of the front kernels, 0 =
+                                   auto (FP64 fronts take 16 columns at most)          */
     uint64_t seed;              /* random sampling seed                                */
     int32_t timing;             /* 1: time every kernel class with CUDA events         */
     int32_t ulv;                /* 1: A_ii of the fronts strictly above the switching
@@ -428,6 +429,10 @@ ndhss_status ndhss_gmres(const ndhss_factorization* f, const int32_t* d_rowptr, 
  * products t = X^T y(I^s), y(B^s) += R(J,:)^T t on the way up and
  * t = R(J,:) z(B^s), z(I^s) += X t on the way down, 32 columns at a time.  A
  * factorization with a ULV diagonal gives INVALID_ARG (ndhss_apply handles it).
+ * Results do not depend on the run, but their last bits depend on the forest:
+ * how a level's products are split (and so the order of their sums, here and in
+ * ndhss_apply with FP64 fronts) follows from how many tasks the level has over
+ * all problems.
  *   nrhs       0..32 right-hand sides
  *   d_x, d_y   device float64 / complex128 (per the factor's vtype) arrays of
  *              n rows, interleaved: element (row, c) at row * ld + c,

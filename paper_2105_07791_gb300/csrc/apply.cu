@@ -638,7 +638,7 @@ __device__ void subtree_task(const ApplyCtx<T>& C, const Entry& e, int* idx, T* 
             const T* A = C.front + foff + (up ? 0 : (int64_t)mi * m) + r;
             const int cols = up ? mi : mb;
             const T* xs = xin + nd[up ? 5 : 7];
-            // rounds of eight loads, the ragged last one predicated: it costs one
+            // rounds of SU loads, the ragged last one predicated: it costs one
             // memory wait, not one per column
             T acc = zero<T>();
             int c = p;

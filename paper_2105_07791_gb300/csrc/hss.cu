@@ -913,6 +913,7 @@ row_id_cluster_kernel(const int* __restrict__ list, const HNode* __restrict__ no
     if (rk == 0 && tid == 0) kk[id] = k;
 }
 
+// Omega_i = X^T Omega_loc, S_i = S_loc(J, :), skeleton = iloc(J).
 template <typename T>
 __global__ void __launch_bounds__(HT)
 finish_kernel(const int* __restrict__ list, const HNode* __restrict__ nodes, const HFront* __restrict__ fronts,
@@ -1197,9 +1198,6 @@ std::vector<HCl> cluster_tree(int n, int top, int beta) {
     return t;
 }
 
-// Stream-ordered scratch (pool allocator): no device-wide synchronisation on
-// allocation or release, uploads from pageable host memory are staged by the
-// runtime before cudaMemcpyAsync returns.
 // Memory for the small host tables of one compression call on one stream: a
 // device block from the pool and a page-locked block, both handed out in
 // order.  The device block starts over with a sampling round (its copies are
@@ -1251,6 +1249,10 @@ struct TableArena {
     }
 };
 
+// Stream-ordered scratch from the pool: no device-wide synchronisation on
+// allocation or release.  An upload lies in the call's TableArena when there is
+// one with room; else it is copied from pageable memory, which the runtime has
+// staged when cudaMemcpyAsync returns.
 template <typename U>
 struct DeviceVec {
     U* p = nullptr;
@@ -1365,7 +1367,7 @@ struct SideFork {
             return set_error(NDHSS_ERR_CUDA, "hss: %s failed: %s", #expr, cudaGetErrorString(e_));           \
     } while (0)
 
-// The batched GEMM of a job list: one launch of 64 x 64 tiles, or, when the
+// The batched GEMM of a job list: one launch of TileShape<T>::GEMM square tiles, or, when the
 // tiles of all jobs leave the GPU mostly idle and K is long, K split over
 // ksplit CTAs per tile plus an ordered reduction of their partials.
 template <typename T, bool RB>

@@ -866,7 +866,7 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
         }
         return pool[pool_next++];
     };
-    std::vector<cudaEvent_t> evs;             // per block: SpMV start, end, apply start, end
+    std::vector<cudaEvent_t> evs;             // per block: SpMV start, its end and the apply's start, apply end
     cudaEvent_t blk_done[2] = {nullptr, nullptr};
     if (cudaEventCreateWithFlags(&blk_done[0], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&blk_done[1], cudaEventDisableTiming) != cudaSuccess)
@@ -877,16 +877,15 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
     for (int blk = 0; blk < max_blocks && rc == NDHSS_OK; ++blk) {
         gm_begin_kernel<V><<<eb, 256, 0, st>>>(S, x, Vb, ldv, t, r, n, blk, (int4*)ctl, nctl);
         note_launches(1);
-        cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr, e3 = nullptr;
-        if (o.timing) { e0 = ev(); e1 = ev(); e2 = ev(); e3 = ev(); }
+        cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
+        if (o.timing) { e0 = ev(); e1 = ev(); e2 = ev(); }
         if (e0) cudaEventRecord(e0, st);
         gm_spmv_kernel<V><<<sblocks, GM_SPT, 0, st>>>(n, rowptr, col, vals, S, b, r, dpart, blk);
         note_launches(1);
         if (e1) cudaEventRecord(e1, st);
-        if (e2) cudaEventRecord(e2, st);
         rc = apply_device(F, 1, nullptr, n, nullptr, n, awork, st, &S->ind);
         if (rc != NDHSS_OK) break;
-        if (e3) cudaEventRecord(e3, st);
+        if (e2) cudaEventRecord(e2, st);
         {
             GmStatus* hs_blk = hst + (blk & 1);
             void* args[] = {(void*)&S, (void*)&Vb, (void*)&ldv, (void*)&n, (void*)&part, (void*)&dpart, (void*)&hs_blk};
@@ -903,7 +902,7 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
             rc = set_error(NDHSS_ERR_CUDA, "ndhss_gmres: launch failed: %s", cudaGetErrorString(le));
             break;
         }
-        if (o.timing) evs.insert(evs.end(), {e0, e1, e2, e3});
+        if (o.timing) evs.insert(evs.end(), {e0, e1, e2});
         cudaEventRecord(blk_done[blk & 1], st);
         nblk = blk + 1;
         if (blk >= 1) {
@@ -938,10 +937,10 @@ ndhss_status gmres_one(const FactorData& F, const int32_t* rowptr, const int32_t
     }
     if (o.timing) {
         float ms;
-        for (int blk = 0; blk < nblk && 4 * blk + 3 < (int)evs.size(); ++blk) {
-            if ((hs.ran[blk] & 1) && cudaEventElapsedTime(&ms, evs[4 * blk], evs[4 * blk + 1]) == cudaSuccess)
+        for (int blk = 0; blk < nblk && 3 * blk + 2 < (int)evs.size(); ++blk) {
+            if ((hs.ran[blk] & 1) && cudaEventElapsedTime(&ms, evs[3 * blk], evs[3 * blk + 1]) == cudaSuccess)
                 Sx.spmv_ms += ms;
-            if ((hs.ran[blk] & 2) && cudaEventElapsedTime(&ms, evs[4 * blk + 2], evs[4 * blk + 3]) == cudaSuccess)
+            if ((hs.ran[blk] & 2) && cudaEventElapsedTime(&ms, evs[3 * blk + 1], evs[3 * blk + 2]) == cudaSuccess)
                 Sx.apply_ms += ms;
         }
     }

@@ -1,14 +1,12 @@
 // Blackwell (sm_100 family) tensor-core primitives as inline PTX: tcgen05 MMA
 // with operands in shared memory and the accumulator in tensor memory (TMEM).
 //
-// Operand layout (K-major, no swizzle): an R x K tile of 32-bit elements is
-// stored as "core matrices" of 8 rows x 16 bytes (128 contiguous bytes, row r
-// at r * 16); core (r / 8, k / 4) sits at ((r / 8) * (K / 4) + k / 4) * 128.
-// The shared-memory descriptor then has leading byte offset 128 (the next
-// core along K) and stride byte offset (K / 4) * 128 (the next 8 rows); one
-// kind::tf32 MMA consumes K = 8, i.e. the start address advances by 256
-// bytes per step.  The accumulator of an M = 128 MMA (cta_group::1) holds row
-// i in TMEM lane i, column j in TMEM column base + j (32-bit each).
+// Operands are K-major tiles that TMA writes with a swizzle (128-byte rows in
+// tcgemm.cu, 64-byte rows in tcgemm64.cu, which build their descriptors): 8-row
+// groups follow each other at the stride byte offset, and a K step of 32 bytes
+// advances the start address by 32 inside the swizzled row.  The accumulator of
+// an M = 128 MMA (cta_group::1) holds row i in TMEM lane i, column j in TMEM
+// column base + j (32-bit each).
 #pragma once
 
 #include <cstdint>
@@ -17,21 +15,6 @@ namespace ndhss {
 namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// byte offset of element (r, k) in a K-major tile of K 32-bit columns
-__device__ __forceinline__ uint32_t core_off(int r, int k, int K) {
-    return ((uint32_t)(r >> 3) * (uint32_t)(K >> 2) + (uint32_t)(k >> 2)) * 128u + (uint32_t)(r & 7) * 16u +
-           (uint32_t)(k & 3) * 4u;
-}
-
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;             // descriptor version of the tcgen05 family
-    return d;                           // base offset 0, no swizzle
-}
 
 // instruction descriptor, kind::tf32: FP32 accumulator, TF32 A and B, both K-major
 __host__ __device__ constexpr uint32_t idesc_tf32(int m, int n) {
@@ -49,13 +32,6 @@ __device__ __forceinline__ uint32_t to_tf32_rn(float v) {
 // MMA share the type), FP32 accumulator, both K-major
 __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
-// byte offset of element (r, k) in a K-major tile of K 16-bit columns: core
-// matrices of 8 rows x 8 elements (16 bytes), LBO 128 (along K), SBO (K / 8) * 128
-__device__ __forceinline__ uint32_t core_off16(int r, int k, int K) {
-    return ((uint32_t)(r >> 3) * (uint32_t)(K >> 3) + (uint32_t)(k >> 3)) * 128u + (uint32_t)(r & 7) * 16u +
-           (uint32_t)(k & 7) * 2u;
 }
 
 // One MMA of kind::f16 (K = 16 for 16-bit operands) or kind::tf32 (K = 8).  The
@@ -93,27 +69,14 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;"); }
-// generic-proxy shared-memory writes become visible to the MMA (async proxy)
-__device__ __forceinline__ void fence_smem_async() { asm volatile("fence.proxy.async.shared::cta;"); }
-
 __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count));
     asm volatile("fence.mbarrier_init.release.cluster;");
 }
 
-// Bounded wait for the given phase parity; false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, int max_iter) {
-    uint32_t done = 0;
-    for (int it = 0; it < max_iter && !done; ++it) {
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(smem_u32(mbar)), "r"(parity));
-    }
-    return done != 0;
-}
-
-// the same without the wait: the values are valid after tmem_wait_ld
+// eight consecutive 32-bit columns of this thread's TMEM lane (warp w reads
+// lanes 32 w .. 32 w + 31: taddr carries the lane offset in bits 16..31), valid
+// after tmem_wait_ld
 __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -123,18 +86,6 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 // (after tmem_wait_ld) keeps the compiler from using the values before the wait
 __device__ __forceinline__ void tmem_landed(uint32_t (&r)[8]) {
     asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
-}
-
-// eight consecutive 32-bit columns of this thread's TMEM lane (warp w reads
-// lanes 32 w .. 32 w + 31: taddr carries the lane offset in bits 16..31)
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(r[u]);
 }
 
 // Bounded waits: how long, and the clock
