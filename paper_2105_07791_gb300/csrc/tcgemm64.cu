@@ -23,7 +23,7 @@
 // Levelling sees to that.  Unknowns on different scales (A -> D A E, D and E
 // diagonal) multiply column q of M'(:, P) by 1 / D_q and row q of M(P, :) by D_q:
 // the products keep their size, but a row's largest entry is that of the pivot
-// with the smallest D_q, and the others lose bits.  tc64_level_kernel reads the
+// with the smallest D_q, and the others lose bits.  pivot_levels reads the
 // pivots' scales off the inverse of their own block, M'(P, P), whose rows all
 // combine every pivot: with r_p the exponent of the largest entry of its row p,
 // column q goes up by s_q = min_p (r_p - exponent of (p, q)) powers of two and
@@ -125,32 +125,33 @@ __device__ __forceinline__ int level_exp(double v, int lev) {
 }
 __device__ __forceinline__ int level_exp(c128 v, int lev) { return max(level_exp(v.x, lev), level_exp(v.y, lev)); }
 
-// The powers of two s_q that level the pivots of an exchange (top of the file),
-// one CTA per front, KW per front in lev: a few KB to read, bound by latency.
+// The powers of two s_q that level the pivots of an exchange (top of the file)
+// into lev, by a CTA of 256 threads.  Every packing CTA forms them itself (64 KB
+// to read from L2 at most, beside its own 32 KB tile and 100 KB of digits): a
+// launch of its own for them took 7 us, 19 -> 26 per exchange.
+template <int KW> struct LevelSmem {
+    int ex[KW][KW + 1];
+    int rmax[KW];
+};
 template <typename T, int KW>
-__global__ void __launch_bounds__(256)
-tc64_level_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front, int k0, int32_t* __restrict__ lev) {
-    __shared__ int ex[KW][KW + 1];
-    __shared__ int rmax[KW];
-    const Front64 P = fronts[blockIdx.x];
-    const int w = P.w;
+__device__ __forceinline__ void pivot_levels(const T* __restrict__ front, const Front64& P, int k0, LevelSmem<KW>& S, int* lev) {
+    const int w = P.w, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const T* D = front + P.foff + (int64_t)k0 * P.m + k0;
-    for (int q = threadIdx.x; q < w * w; q += 256) ex[q % w][q / w] = level_exp(D[(int64_t)(q / w) * P.m + q % w], 0);
+    for (int q = threadIdx.x; q < w * w; q += 256) S.ex[q % w][q / w] = level_exp(D[(int64_t)(q / w) * P.m + q % w], 0);
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int p = warp; p < w; p += 8) {
         int r = INT_MIN;
-        for (int q = lane; q < w; q += 32) r = max(r, ex[p][q]);
+        for (int q = lane; q < w; q += 32) r = max(r, S.ex[p][q]);
         r = __reduce_max_sync(0xffffffffu, r);
-        if (lane == 0) rmax[p] = r;
+        if (lane == 0) S.rmax[p] = r;
     }
     __syncthreads();
     for (int q = warp; q < w; q += 8) {
         int s = INT_MAX;
         for (int p = lane; p < w; p += 32)
-            if (ex[p][q] != INT_MIN) s = min(s, rmax[p] - ex[p][q]);
+            if (S.ex[p][q] != INT_MIN) s = min(s, S.rmax[p] - S.ex[p][q]);
         s = __reduce_min_sync(0xffffffffu, s);
-        if (lane == 0) lev[(int64_t)blockIdx.x * KW + q] = s == INT_MAX ? 0 : min(s, 4096);
+        if (lane == 0) lev[q] = s == INT_MAX ? 0 : min(s, 4096);
     }
 }
 
@@ -167,13 +168,17 @@ __device__ __forceinline__ float next_digit(int64_t& x, bool last) {
 // the pivots; pivots from w on are zeros.
 template <typename T, int KW>
 __global__ void __launch_bounds__(256)
-tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front, const int32_t* __restrict__ lev, int k0,
-                 int j0, __nv_bfloat16* __restrict__ packed, int32_t* __restrict__ rexp) {
+tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front, int k0, int j0,
+                 __nv_bfloat16* __restrict__ packed, int32_t* __restrict__ rexp) {
     constexpr bool CPLX = Tr<T>::cplx;
     constexpr int CX = CPLX ? 2 : 1;
     constexpr int Kp = packed_k<T, KW>(), KL = Kp / CX;      // packed values and entries of a row
     constexpr int LPR = KL < 32 ? KL : 32, UL = KL / LPR, RW = 32 / LPR;
-    __shared__ T ts[32][KL + 1];
+    // the levels' scratch, then the tile
+    constexpr size_t TS = sizeof(T) * 32 * (KL + 1);
+    __shared__ __align__(16) unsigned char sm[TS > sizeof(LevelSmem<KW>) ? TS : sizeof(LevelSmem<KW>)];
+    __shared__ int s_lev[KW];
+    T (*ts)[KL + 1] = reinterpret_cast<T(*)[KL + 1]>(sm);
     const Front64 P = fronts[blockIdx.y];
     const int m = P.m, w = P.w, nb = P.nb;
     const int rt_a = (m + 31) / 32, rt_b = (nb + 31) / 32;
@@ -182,6 +187,8 @@ tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front
     const int r0 = ((int)blockIdx.x - (is_a ? 0 : rt_a)) * 32, rows = is_a ? m : nb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane / LPR, ll = lane % LPR;
     const T* F = front + P.foff;
+    pivot_levels<T, KW>(front, P, k0, *reinterpret_cast<LevelSmem<KW>*>(sm), s_lev);
+    __syncthreads();
     if (is_a) {
         for (int l = warp; l < KL; l += 8) {
             const int r = r0 + lane;
@@ -203,7 +210,7 @@ tc64_pack_kernel(const Front64* __restrict__ fronts, const T* __restrict__ front
 #pragma unroll
     for (int u = 0; u < UL; ++u) {
         const int l = ll + LPR * u;
-        const int s = l < w ? lev[(int64_t)blockIdx.y * KW + l] : 0;
+        const int s = l < w ? s_lev[l] : 0;
         lv[u] = is_a ? s : -s;
     }
     for (int rr = RW * warp + sub; rr < 32; rr += 8 * RW) {
@@ -538,10 +545,9 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
             rt_max = std::max(rt_max, (m + 31) / 32 + (nb + 31) / 32);
         }
         if (fr.empty()) break;
-        // one pool allocation: packed digits, row exponents and the pivots'
-        // levels, then the tables
+        // one pool allocation: packed digits, row exponents, then the tables
         auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
-        const size_t packed_bytes = r256((size_t)rows * Kp * 2), exp_bytes = packed ? r256(((size_t)nexp + fr.size() * KW) * 4) : 0;
+        const size_t packed_bytes = r256((size_t)rows * Kp * 2), exp_bytes = packed ? r256((size_t)nexp * 4) : 0;
         const size_t fr_bytes = r256(fr.size() * sizeof(Front64)), job_bytes = r256(jobs.size() * sizeof(Job64));
         const size_t t_bytes = r256(tiles.size() * sizeof(int2));
         std::vector<unsigned char> tab(fr_bytes + job_bytes + t_bytes);
@@ -558,7 +564,6 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
             continue;
         }
         int32_t* d_exp = reinterpret_cast<int32_t*>(buf + packed_bytes);
-        int32_t* d_lev = d_exp + nexp;
         unsigned char* d_tab = buf + packed_bytes + exp_bytes;
         const Front64* d_fr = reinterpret_cast<const Front64*>(d_tab);
         T* front = static_cast<T*>(F.d_front);
@@ -596,12 +601,8 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
                                   CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (rc == NDHSS_OK) {
-            tc64_level_kernel<T, KW><<<(unsigned)fr.size(), 256, 0, st>>>(d_fr, front, k0, d_lev);
-            launched("tc64_level_kernel");
-        }
-        if (rc == NDHSS_OK) {
             tc64_pack_kernel<T, KW><<<dim3((unsigned)rt_max, (unsigned)fr.size()), 256, 0, st>>>(
-                d_fr, front, d_lev, k0, j0, reinterpret_cast<__nv_bfloat16*>(buf), d_exp);
+                d_fr, front, k0, j0, reinterpret_cast<__nv_bfloat16*>(buf), d_exp);
             launched("tc64_pack_kernel");
         }
         if (rc == NDHSS_OK) {
