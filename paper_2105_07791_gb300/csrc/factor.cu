@@ -1161,7 +1161,8 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
         // every other column of the front.  The arithmetic is the sweep's own
         // (a block of exchanges composed), so S stays the elimination's Schur
         // complement.  Small fronts keep the rank-kb steps over the whole front.
-        const bool tcl = tc_front_path(F, mimax);
+        const TcPath path = tc_front_path(F, nodes, mimax);
+        const bool tcl = path.blocks, inner = path.inner;
         const int okb = F.prec == NDHSS_FP64 ? TC64_KB2 : TC_KB2;
         const int kb2 = tcl ? okb : 0;
         const int gt = (int)((mmax + GT - 1) / GT);
@@ -1170,7 +1171,6 @@ ndhss_status factor_run(FactorData& F, const Tree& t, const V* d_vals, const int
         // exchanged on the tensor cores too (tc64_block_exchange with the panel as
         // its pivots), so the FP64 pipe updates the panel's own columns only (256 x
         // 256 P2 Helmholtz, complex128: updates 50 -> 23 ms, exchanges 24 -> 41).
-        const bool inner = tcl && F.prec == NDHSS_FP64 && mimax >= TC64_INNER_MIN;
         const int pgx = (int)std::min<int64_t>({(mmax + PREP_WARPS - 1) / PREP_WARPS, 1024,
                                                 std::max<int64_t>(1, PREP_CTAS / std::max(1, std::min(L, MAX_GRID_YZ)))});
         for (int64_t k0 = 0; k0 < mimax;) {

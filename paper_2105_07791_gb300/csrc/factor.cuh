@@ -153,9 +153,16 @@ constexpr int TC_KB2 = 128;
 constexpr int TC64_KB2 = 64;     // the same for FP64 fronts (tcgemm64.cu)
 constexpr int TC64_KB1 = 16;     // widest panel exchanged inside an outer block of FP64 fronts
 constexpr int TC64_INNER_MIN = 64;   // from this largest interior block of a level on
+// How a level is swept: in outer blocks exchanged on the tensor cores, and
+// (FP64) whether the panels' exchanges inside a block run there too.
+struct TcPath {
+    bool blocks, inner;
+};
 // Whether a level whose largest interior block has mi_max unknowns takes the
-// two-level sweep with tensor-core block exchanges; tcgemm.cu.
-bool tc_front_path(const FactorData& F, int64_t mi_max);
+// two-level sweep with tensor-core block exchanges; tcgemm.cu, FP64 fronts
+// tcgemm64.cu (`forced`: the interior block's size alone decides).
+TcPath tc_front_path(const FactorData& F, const std::vector<int>& nodes, int64_t mi_max);
+TcPath tc64_front_path(const FactorData& F, const std::vector<int>& nodes, int64_t mi_max, bool forced);
 // The exchange of the outer pivot block starting at pivot k0 (its slab of
 // columns [k0, k0 + TC_KB2) already swept, the row interchanges applied to
 // every column) on every other column of the fronts of `nodes`, as one

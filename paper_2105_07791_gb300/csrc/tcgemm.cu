@@ -564,16 +564,17 @@ ndhss_status tc_block_t(FactorData& F, const std::vector<int>& nodes, int k0, De
 
 }  // namespace
 
-bool tc_front_path(const FactorData& F, int64_t mi_max) {
+TcPath tc_front_path(const FactorData& F, const std::vector<int>& nodes, int64_t mi_max) {
     // NDHSS_TC_MIN_MI: smallest largest-interior-block of a level that takes
     // the two-level sweep (default 96; smaller fronts leave the blocks and
     // 128 x 128 tiles mostly empty); NDHSS_FRONT_UPDATE=simt keeps every
     // level on the rank-kb sweep over whole fronts (CUDA cores; a cross-check)
     const char* u = std::getenv("NDHSS_FRONT_UPDATE");
-    if (u && std::strcmp(u, "simt") == 0) return false;
+    if (u && std::strcmp(u, "simt") == 0) return {false, false};
     const char* e = std::getenv("NDHSS_TC_MIN_MI");
     const int min_mi = e ? std::atoi(e) : F.prec == NDHSS_FP64 ? 24 : 96;
-    return min_mi > 0 && mi_max >= min_mi;
+    if (min_mi <= 0 || mi_max < min_mi) return {false, false};
+    return F.prec == NDHSS_FP64 ? tc64_front_path(F, nodes, mi_max, e != nullptr) : TcPath{true, false};
 }
 
 ndhss_status tc_block_exchange(FactorData& F, const std::vector<int>& nodes, int k0, DevStatus* d_status,

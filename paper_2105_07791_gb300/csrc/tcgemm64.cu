@@ -620,6 +620,27 @@ ndhss_status tc64_block_run(FactorData& F, const std::vector<int>& nodes, int k0
 
 }  // namespace
 
+// Complex fronts: blocks from 24 interior unknowns on, panels from 64 on.  A
+// rank-16 update of a 64 x 64 tile holds an SM's FP64 pipe for 64 us there, more
+// than the launches of an exchange cost (some 20 us).  Real fronts: 16 us, so the
+// exchanges pay only where a level has more tiles than SMs.  A level whose rank-16
+// updates fill less than two waves stays on the CUDA cores unless its pivots go in
+// several blocks (96 unknowns), and the panels are exchanged in blocks whose
+// slabs, one 64-column tile per 64 rows, fill one and a half.
+TcPath tc64_front_path(const FactorData& F, const std::vector<int>& nodes, int64_t mi_max, bool forced) {
+    if (F.vtype == NDHSS_C128 || forced) return {true, mi_max >= TC64_INNER_MIN};
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int64_t slab = 0, all = 0;                      // 64 x 64 tiles of a slab's and of a whole level's update
+    for (int s : nodes) {
+        const int64_t t = F.m_i(s) > 0 ? (F.m_i(s) + F.m_b(s) + 63) / 64 : 0;
+        slab += t;
+        all += t * t;
+    }
+    const bool blocks = mi_max >= 96 || all >= 2 * sms;
+    return {blocks, blocks && mi_max >= TC64_INNER_MIN && 2 * slab >= 3 * sms};
+}
+
 ndhss_status tc64_block_exchange(FactorData& F, const std::vector<int>& nodes, int k0, int width, int j0, int j1,
                                  DevStatus* d_status, cudaStream_t st) {
     // the packed width by the call's widest pivot block

@@ -28,7 +28,8 @@ def nd():
 
 @pytest.mark.parametrize("kind", ["poisson", "helmholtz"])
 @pytest.mark.parametrize("e", [-1000, -960, 960, 1005])
-def test_factor_of_a_matrix_scaled_to_the_ends_of_the_range(nd, kind, e):
+def test_factor_of_a_matrix_scaled_to_the_ends_of_the_range(nd, kind, e, monkeypatch):
+    monkeypatch.setenv("NDHSS_TC_MIN_MI", "24")       # small levels too, real and complex
     P = poisson_dirichlet(40, p=2, seed=2) if kind == "poisson" else helmholtz_impedance(40, 2, 16.0, seed=2)
     tree = nd.ndhss_build_tree(P.coords, P.A.indptr, P.A.indices, 64)
     x = torch.from_numpy(np.random.default_rng(0).standard_normal(P.n).astype(P.A.dtype)).cuda()

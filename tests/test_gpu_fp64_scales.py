@@ -54,7 +54,8 @@ def _cabs(a):
 
 @pytest.mark.parametrize("kind", ["poisson", "poisson_p2", "helmholtz"])
 @pytest.mark.parametrize("s,both", [(0, True), (24, True), (48, True), (80, True), (40, False)])
-def test_exchange_matches_extended_precision(nd, kind, s, both):
+def test_exchange_matches_extended_precision(nd, kind, s, both, monkeypatch):
+    monkeypatch.setenv("NDHSS_TC_MIN_MI", "24")       # small levels too, real and complex
     P, leaf = _problem(kind)
     rng = np.random.default_rng(s)
     Dr = np.exp2(rng.uniform(0, s, P.n))
@@ -99,6 +100,7 @@ def test_entries_that_are_not_finite_end_as_in_the_cuda_core_sweep(nd, kind, bad
     """One such entry: the same status from both sweeps, or results that are not
     finite in both, or (an infinite pivot has the inverse zero) finite ones that
     agree to rounding (2^-53) times the condition number (2^17 here)."""
+    monkeypatch.setenv("NDHSS_TC_MIN_MI", "24")
     P, leaf = _problem(kind)
     A = sp.csr_matrix(P.A).copy()
     row = P.n // 2

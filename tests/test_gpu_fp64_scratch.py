@@ -75,6 +75,7 @@ def test_smaller_batches_and_fronts_without_packed_operands(nd, kind, p, limit, 
     """Batches change no product (bit for bit, as long as every front fits one);
     fronts without packed operands take float64 ones: rounding times the
     condition number (2^17 at most here)."""
+    monkeypatch.setenv("NDHSS_TC_MIN_MI", "24")       # small levels too, real and complex
     N = 96 // p + 5
     P = poisson_dirichlet(N, p=p, seed=2) if kind == "poisson" else helmholtz_impedance(N, p, 12.0, seed=2)
     tree = nd.ndhss_build_tree(P.coords, P.A.indptr, P.A.indices, 64)
