@@ -1609,15 +1609,24 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
     // (four per SM) take FINE_ROWS: their time is the FP64 pipe's, so it is the
     // number of SMs with work that counts (one apply, 256 x 256 P2 Helmholtz,
     // dense complex128, 1.45 GB: 1571 us with 64 rows everywhere, 1005 so; all
-    // levels fine is 1079).
+    // levels fine is 1079).  Tasks of few columns are done before that pays (64
+    // rows x 64 real or 32 complex columns take 1 or 2 us): 40 x 40 Helmholtz in
+    // leaves of 12 unknowns 158 us with 16 rows at any width, 132 so (136 with 64
+    // rows everywhere); 250 x 250 Poisson 146 and 137.
     constexpr int FINE_TASKS = 4 * 152;
-    auto pick_rows = [&](int64_t tasks) { return F.prec == NDHSS_FP64 && tasks < FINE_TASKS ? FINE_ROWS : APPLY_ROWS; };
+    const int fine_cols = F.vtype == NDHSS_C128 ? 32 : 64;
+    auto pick_rows = [&](int64_t tasks, int cols) {
+        return F.prec == NDHSS_FP64 && tasks < FINE_TASKS && cols >= fine_cols ? FINE_ROWS : APPLY_ROWS;
+    };
     std::vector<int> rows_up(F.depth + 1, APPLY_ROWS), rows_dn(F.depth + 1, APPLY_ROWS);
     for (int l = 0; l <= l_top; ++l) {
         int64_t up = 0, dn = 0;
+        int cup = 0, cdn = 0;                      // columns of the widest task
         for (int s : F.levels[l]) {
             const int mi = F.m_i(s), mb = F.m_b(s);
             if (mi == 0) continue;
+            cup = std::max(cup, std::min(mi, DIAG_COLS));
+            cdn = std::max(cdn, mb);
             if (fused(s)) {
                 up += ceil_div(mi + mb, APPLY_ROWS);
             } else {
@@ -1626,8 +1635,8 @@ ndhss_status build_apply_schedule(FactorData& F, cudaStream_t st) {
             }
             if (mode(s) == 0) dn += ceil_div(mi, APPLY_ROWS);
         }
-        rows_up[l] = pick_rows(up);
-        rows_dn[l] = pick_rows(dn);
+        rows_up[l] = pick_rows(up, cup);
+        rows_dn[l] = pick_rows(dn, cdn);
     }
     auto push_dpart = [&](int l) {
         for (int s : F.levels[l]) {
