@@ -71,7 +71,7 @@ struct FactorData {
     // each level's range in both
     int2* d_mjobs = nullptr;
     std::vector<int64_t> mj_up_off, mj_dn_off;
-    std::vector<int64_t> mj_up_tiles, mj_dn_tiles;   // 32-row tiles per level
+    std::vector<char> mj_up_deep, mj_dn_deep;        // per level: K split over four thread groups
     // low-rank nodes of the multi apply: (node, first row, T offset) tiles
     // per level of the four products t = X^T u(I), u(B) += RJt t,
     // t = RJt^T z(B), z(I) += X t; T scratch elements (k x 32 per node)

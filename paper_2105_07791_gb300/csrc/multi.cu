@@ -39,7 +39,11 @@ constexpr int MR = 32;            // interleaved right-hand sides
 constexpr int MT_ROWS = 64;       // rows per apply tile
 constexpr int MT_K = 16;          // K chunk of an apply tile
 constexpr int MT_THREADS = 128;   // threads of a dense apply tile (4 x 4 products each)
-constexpr int MT_DEEP = 4 * 152;  // levels with fewer 32-row tiles split K over four groups
+// Levels with fewer 32-row tiles than MT_DEEP split K over four groups; those with
+// a tile per SM (MT_FEW) only if a sum is longer than two chunks, else the groups'
+// barriers cost more than they save (200 problems of 6 to 10 cells, leaves of 24:
+// 90 us with one group, 107 with four, 93 so).
+constexpr int MT_DEEP = 4 * 152, MT_FEW = 152;
 constexpr int MF_ROWS = 8, MF_COLS = 4, MF_THREADS = 128;   // FP64 apply: outputs per CTA, four warps over K
 constexpr int SEG_ROWS = 1024;    // rows per reduction block
 // The row-wise kernels (product, vector updates) split a reduction block over
@@ -464,7 +468,7 @@ ndhss_status multi_apply_run(const FactorData& F, int nrhs, const V* X, int64_t 
                 else
                     mapply_fp64_kernel<T, false><<<grid, MF_THREADS, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
             } else {
-                const bool deep = (up ? F.mj_up_tiles : F.mj_dn_tiles)[l] < MT_DEEP;
+                const bool deep = (up ? F.mj_up_deep : F.mj_dn_deep)[l] != 0;
                 auto launch = [&](auto kernel, int threads) {
                     kernel<<<(unsigned)(b - a), threads, 0, st>>>(jb, F.d_node, F.d_foff, front, F.d_sigma, F.d_blist, U, Z, pact, nprob, lrp);
                 };
@@ -1117,15 +1121,24 @@ ndhss_status build_multi_plan(FactorData& F, cudaStream_t st) {
     F.mj_up_off[2 * (F.depth + 1)] = (int64_t)jobs.size() / 2;
     // 32-row tiles per level, whatever shape the jobs have (the summation order
     // depends on it, and must not on the shape)
-    F.mj_up_tiles.assign(F.depth + 1, 0);
-    F.mj_dn_tiles.assign(F.depth + 1, 0);
-    for (int l = 0; l <= F.depth; ++l)
+    F.mj_up_deep.assign(F.depth + 1, 0);
+    F.mj_dn_deep.assign(F.depth + 1, 0);
+    for (int l = 0; l <= F.depth; ++l) {
+        int64_t up = 0, dn = 0;
+        int kup = 0, kdn = 0;                        // longest sums of the level
         for (int s : F.levels[l]) {
             const int mi = F.m_i(s), mb = F.m_b(s);
             if (mi == 0) continue;
-            F.mj_up_tiles[l] += ((lowrank(s) ? mi : mi + mb) + 31) / 32;
-            if (mb > 0 && !lowrank(s)) F.mj_dn_tiles[l] += (mi + 31) / 32;
+            up += ((lowrank(s) ? mi : mi + mb) + 31) / 32;
+            kup = std::max(kup, mi);
+            if (mb > 0 && !lowrank(s)) {
+                dn += (mi + 31) / 32;
+                kdn = std::max(kdn, mb);
+            }
         }
+        F.mj_up_deep[l] = up < MT_DEEP && (up < MT_FEW || kup > 2 * MT_K);
+        F.mj_dn_deep[l] = dn < MT_DEEP && (dn < MT_FEW || kdn > 2 * MT_K);
+    }
     for (int l = 0; l <= F.depth; ++l)
         for (int v = 0; v < 2; ++v) {
             F.mj_dn_off[2 * l + v] = (int64_t)jobs.size() / 2;
