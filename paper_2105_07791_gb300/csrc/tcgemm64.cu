@@ -30,10 +30,11 @@
 // row q of M down by as many (exact: exponents only).  Errors of one exchange
 // relative to D_i E_j, scales over 2^24 / 2^48 / 2^80: 1e-11 / 6e-5 / 1 without
 // levelling, 1e-16 / 7e-16 / 5e-16 with it, 4e-16 in float64.
-//  The epilogue joins the eight integers into two of 51 bits in
-// integer arithmetic, those into one float64 value rounded once (two FMAs,
-// ints_scaled) and adds it to the front: three FP64 instructions per element
-// (summing the eight in float64 would make the FP64 pipe the bound again).
+//
+// The epilogue joins the eight integers into two of 51 bits in integer
+// arithmetic, those into one float64 value rounded once (two FMAs, ints_scaled)
+// and adds it to the front: three FP64 instructions per element (summing the
+// eight in float64 would make the FP64 pipe the bound again).
 //
 // Rows with an infinity or a NaN give NaN.
 //
